@@ -181,9 +181,10 @@ salec_status salec_step(salec_ctx* ctx, int nsteps);
  *                      every phase returns its input, only reads and writes its state.
  *                      A tile found quiescent in the step before, with its eight
  *                      neighbours, is at rest: it is copied without a halo (by a
- *                      streaming kernel before the tile kernel, or by a copy kernel
- *                      beside it: salec_set_rest_copy), and the other tiles are queued
- *                      for the tile kernel (one CTA per resident slot of the device).
+ *                      streaming kernel before the tile kernel, once for as long as it
+ *                      stays at rest, or by a copy kernel beside it, every step:
+ *                      salec_set_rest_copy), and the other tiles are queued for the tile
+ *                      kernel (one CTA per resident slot of the device).
  *                      Default when grid->gravity == 0.
  *   SALEC_STEP_PHASES  six kernels over the whole grid and the Courant kernel, in place
  *                      (block shapes from salec_set_block_shapes / salec_autotune).
@@ -201,7 +202,8 @@ int salec_get_step_form(const salec_ctx* ctx);
  * after set-up, a host write or other steps, when the Courant-rate pass over that state
  * found them quiescent with fields already in the form the quiescent path writes).
  *   mode 0  every tile goes through the tile kernel;
- *   mode 1  (default) a streaming kernel copies the tiles at rest and queues the others
+ *   mode 1  (default) a streaming kernel copies the tiles newly at rest (a tile that stays
+ *           at rest is then the same in both copies of the fields) and queues the others
  *           before the tile kernel starts;
  *   mode 2  a scan kernel queues the tiles, and a copy kernel of one warp per SM
  *           on a second stream of the context moves the tiles at rest with bulk tensor

@@ -45,6 +45,7 @@ struct Layout {
     size_t rest[2];   // the fused form's rest flags of the tiles, one per copy
     size_t work;      // two TileWork queues (one per copy the step reads)
     size_t list;      // the queued tiles
+    size_t rest_rate; // the Courant rates of the tiles at rest
     size_t ntiles;    // bound on the fused form's tile count
     size_t total;
 };
@@ -121,6 +122,7 @@ Layout make_layout(const salec_grid& g, int precision)
     L.rest[1] = take(cur, L.ntiles);
     L.work = take(cur, 2 * sizeof(TileWork));
     L.list = take(cur, L.ntiles * sizeof(int));
+    L.rest_rate = take(cur, L.ntiles * sizeof(unsigned long long));
     size_t nb = 0;
     for (int k = 0; k < kNumShapes; ++k) {
         const size_t t = (size_t)tiles_of(g.nr, g.nz, 0, kShapes[k]);
@@ -309,6 +311,7 @@ static void fill_pingpong(salec_ctx* ctx, const ParamsT<T>& P0, ParamsT<T>& P1, 
         o.work = at<TileWork>(ctx, L.work) + k;
         o.work_next = at<TileWork>(ctx, L.work) + w;
         o.list = at<int>(ctx, L.list);
+        o.rest_rate = at<unsigned long long>(ctx, L.rest_rate);
     }
 }
 

@@ -1023,6 +1023,22 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
     }
 }
 
+// A tile is at rest when it and its eight neighbours (those inside the grid) took the
+// quiescent path in the step that wrote the copy read here.
+__device__ __forceinline__ bool tile_at_rest(const unsigned char* __restrict__ rest_in, int tile, int nbx, int nby)
+{
+    const int bx = tile % nbx, by = tile / nbx;
+    int rest = 1;
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+        for (int dx = -1; dx <= 1; ++dx) {
+            const int tx = bx + dx, ty = by + dy;
+            if (tx >= 0 && tx < nbx && ty >= 0 && ty < nby) rest &= rest_in[ty * nbx + tx] != 0;
+        }
+    return rest != 0;
+}
+
 // ---- tiles at rest.  A tile that the step before took through the quiescent path, and
 // whose eight neighbours it took through it too, has an unchanged frame that still passes
 // every test of that path; and its fields already are what that path writes (an absent
@@ -1030,10 +1046,22 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
 // So its outputs are its inputs bit for bit, its peak over-pressure stays (the same
 // pressure against the same reference as in the step before), and its Courant rate is
 // that of its fastest sound speed: one square root of the largest c^2 of its cells on a
-// uniform grid (the rounded square root is monotonic).  This kernel copies those tiles,
-// one warp per tile with the loads of several rows in flight, and queues every other tile
-// for the tile kernel.
-constexpr int kRestThreads = 256;
+// uniform grid (the rounded square root is monotonic).
+//
+// A tile at rest is copied once.  After a step has copied it, both copies of the fields
+// hold it, so the next step, which writes the copy this one read, finds its outputs already
+// there as long as the tile stays at rest: it then only enters the tile's Courant rate, kept
+// with the flags (rest flag 2, rest_rate).  Anything that changes the fields other than a
+// fused step starts again from flags of 1 (the Courant-rate pass), and bringing the second
+// copy home makes the two copies the same.  Moving the tiles at rest at every step took
+// 0.215 ms (FP64, 96 % of the measured copy bandwidth) and 0.130 ms (mixed) of a 4000 x 4000
+// step; testing the flags takes the place of it.
+//
+// A block of eight warps tests 32 tiles, one lane a tile: its first warp enters the kept
+// rates and queues the tiles that are not at rest (one atomic a warp and end of the list);
+// the tiles to copy are dealt to the eight warps, each with the loads of several rows in
+// flight.
+constexpr int kRestThreads = 256, kRestTiles = 32;
 
 template <typename T, int NM, bool STR, bool UNI, int TW, int TH>
 __global__ void __launch_bounds__(kRestThreads) k_rest_tiles(const ParamsT<T> P, const OutPtrsT<T> O)
@@ -1046,107 +1074,142 @@ __global__ void __launch_bounds__(kRestThreads) k_rest_tiles(const ParamsT<T> P,
     const PtrsT<T>& p = P.p;
     const T zero = T(0);
     const int nr = P.nr, nz = P.nz, nv = nr + 1;
-    const int nbx = (nr + TW - 1) / TW, nby = (nz + TH - 1) / TH;
+    const int nbx = (nr + TW - 1) / TW, nby = (nz + TH - 1) / TH, ntiles = nbx * nby;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int tile = blockIdx.x * (kRestThreads / 32) + w;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         O.work_next->count = 0;
         O.work_next->next = 0;
         O.work_next->back = 0;
         O.work_next->copy_next = 0;
     }
-    T c2max = zero, speed_max = zero;
-    bool bad = false;
-    if (tile < nbx * nby) {
-        const int bx = tile % nbx, by = tile / nbx;
-        bool rest = true;
-        if (lane < 9) {
-            const int tx = bx + lane % 3 - 1, ty = by + lane / 3 - 1;
-            if (tx >= 0 && tx < nbx && ty >= 0 && ty < nby) rest = O.rest_in[ty * nbx + tx] != 0;
+    // the block's tiles, one a lane (every warp tests all of them)
+    const int mine = blockIdx.x * kRestTiles + lane;
+    const int flag = mine < ntiles ? O.rest_in[mine] : 0;
+    const bool rest = mine < ntiles && tile_at_rest(O.rest_in, mine, nbx, nby);
+    const unsigned copies = __ballot_sync(0xffffffffu, rest && flag != 2);
+    unsigned long long bits = 0ull;
+    if (w == 0) {
+        if (rest && flag == 2) {
+            O.rest_out[mine] = 2;
+            bits = O.rest_rate[mine];
         }
-        rest = __all_sync(0xffffffffu, rest);
-        if (!rest) {
-            // each tile is queued once a step: one that took the whole cycle in the step
-            // before at the front, one queued only for a neighbour (most of these take the
-            // quiescent path again) at the back, so that the long cycles start first and
-            // the short ones fill the end of the kernel
-            if (lane == 0) {
-                if (O.rest_in[tile] == 0) {
-                    const int q = atomicAdd(&O.work->count, 1);
-                    if (q < nbx * nby) O.list[q] = tile;
-                } else {
-                    const int q = atomicAdd(&O.work->back, 1);
-                    if (q < nbx * nby) O.list[nbx * nby - 1 - q] = tile;
-                }
-            }
-        } else {
-            if (lane == 0) O.rest_out[tile] = 1;
-            const int i = bx * TW + lane, jb = by * TH, je = min(jb + TH, nz);
-            if (i < nr) {
-                for (int j0 = jb; j0 < je; j0 += R) {
-                    T2 fr[R][NM], ec[R], sd[R];
-                    double Ic[R];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        if (j0 + r >= je) break;
-                        const int c = (j0 + r) * nr + i;
-#pragma unroll
-                        for (int m = 0; m < NM; ++m) fr[r][m] = p.fr[m][c];
-                        Ic[r] = p.I[c];
-                        ec[r] = p.eosc[c];
-                        if (STR) sd[r] = p.s2d[c];
-                    }
-#pragma unroll
-                    for (int r = 0; r < R; ++r) {
-                        if (j0 + r >= je) break;
-                        const int j = j0 + r, c = j * nr + i;
-                        bool here = false;
-#pragma unroll
-                        for (int m = 0; m < NM; ++m) {
-                            O.fr[m][c] = fr[r][m];
-                            here = here || pos(fr[r][m].x);
-                        }
-                        O.I[c] = Ic[r];
-                        O.eosc[c] = ec[r];
-                        if (STR) {
-                            O.s01[c] = V::mk(zero, zero);
-                            O.s2d[c] = sd[r];
-                        }
-                        if (here) {
-                            const T c2 = ec[r].y;
-                            if (!UNI || is_nan(c2) || neg(c2)) {
-                                // the quiescent path's own arithmetic, cell by cell
-                                T speed = t_sqrt<T>(zero) + t_sqrt<T>(c2);
-                                if (!UNI) speed = speed * GE::ilen(P, i, j);
-                                bad = bad || is_nan(speed);
-                                speed_max = max_nonneg(speed_max, speed);
-                            } else {
-                                c2max = max_nonneg(c2max, c2);
-                            }
-                        }
-                    }
-                }
-            }
-            // the tile's vertices (with the grid's far edges on the last tiles) at rest
-            const int jv = by == nby - 1 ? nz + 1 : jb + TH;
-            const bool edge = lane == 0 && bx == nbx - 1 && bx * TW + TW == nr;
-            for (int j = jb; j < jv; ++j) {
-                if (i <= nr) O.v[j * nv + i] = V::mk(zero, zero);
-                if (edge) O.v[j * nv + nr] = V::mk(zero, zero);
-            }
+        // each tile is queued once a step: one that took the whole cycle in the step before
+        // at the front, one queued only for a neighbour (most of these take the quiescent
+        // path again) at the back, so that the long cycles start first and the short ones
+        // fill the end of the kernel
+        const bool queue = mine < ntiles && !rest;
+        const unsigned below = (1u << lane) - 1u;
+        const unsigned front = __ballot_sync(0xffffffffu, queue && flag == 0);
+        const unsigned back = __ballot_sync(0xffffffffu, queue && flag != 0);
+        int qf = 0, qb = 0;
+        if (lane == 0) {
+            if (front) qf = atomicAdd(&O.work->count, __popc(front));
+            if (back) qb = atomicAdd(&O.work->back, __popc(back));
+        }
+        qf = __shfl_sync(0xffffffffu, qf, 0) + __popc(front & below);
+        qb = __shfl_sync(0xffffffffu, qb, 0) + __popc(back & below);
+        if (front >> lane & 1u) {
+            if (qf < ntiles) O.list[qf] = mine;
+        } else if (back >> lane & 1u) {
+            if (qb < ntiles) O.list[ntiles - 1 - qb] = mine;
         }
     }
-    if (UNI) speed_max = max_nonneg(speed_max, t_sqrt<T>(zero) + t_sqrt<T>(c2max));
+    // the tiles to copy, dealt to the warps in turn
+    bool bad = false;
+    int nth = 0;
+    for (unsigned left = copies; left; left &= left - 1u, ++nth) {
+        if (nth % (kRestThreads / 32) != w) continue;
+        const int tile = blockIdx.x * kRestTiles + __ffs(left) - 1;
+        const int bx = tile % nbx, by = tile / nbx;
+        T c2max = zero, speed_max = zero;
+        // the copy writes vertices at rest and no deviatoric stress as +0: the tile is the
+        // same in both copies if the copy read has no -0 there (else after the next copy)
+        bool same = true;
+        const int i = bx * TW + lane, jb = by * TH, je = min(jb + TH, nz);
+        if (i < nr) {
+            for (int j0 = jb; j0 < je; j0 += R) {
+                T2 fr[R][NM], ec[R], sd[R], ss[R];
+                double Ic[R];
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (j0 + r >= je) break;
+                    const int c = (j0 + r) * nr + i;
+#pragma unroll
+                    for (int m = 0; m < NM; ++m) fr[r][m] = p.fr[m][c];
+                    Ic[r] = p.I[c];
+                    ec[r] = p.eosc[c];
+                    if (STR) {
+                        sd[r] = p.s2d[c];
+                        ss[r] = p.s01[c];
+                    }
+                }
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    if (j0 + r >= je) break;
+                    const int j = j0 + r, c = j * nr + i;
+                    bool here = false;
+#pragma unroll
+                    for (int m = 0; m < NM; ++m) {
+                        O.fr[m][c] = fr[r][m];
+                        here = here || pos(fr[r][m].x);
+                    }
+                    O.I[c] = Ic[r];
+                    O.eosc[c] = ec[r];
+                    if (STR) {
+                        O.s01[c] = V::mk(zero, zero);
+                        O.s2d[c] = sd[r];
+                        same = same && is_pzero(ss[r].x) && is_pzero(ss[r].y);
+                    }
+                    if (here) {
+                        const T c2 = ec[r].y;
+                        if (!UNI || is_nan(c2) || neg(c2)) {
+                            // the quiescent path's own arithmetic, cell by cell
+                            T speed = t_sqrt<T>(zero) + t_sqrt<T>(c2);
+                            if (!UNI) speed = speed * GE::ilen(P, i, j);
+                            bad = bad || is_nan(speed);
+                            speed_max = max_nonneg(speed_max, speed);
+                        } else {
+                            c2max = max_nonneg(c2max, c2);
+                        }
+                    }
+                }
+            }
+        }
+        // the tile's vertices (with the grid's far edges on the last tiles) at rest
+        const int jv = by == nby - 1 ? nz + 1 : jb + TH;
+        const bool edge = lane == 0 && bx == nbx - 1 && bx * TW + TW == nr;
+        for (int j = jb; j < jv; ++j) {
+            if (i <= nr) {
+                const T2 v = p.v[j * nv + i];
+                same = same && is_pzero(v.x) && is_pzero(v.y);
+                O.v[j * nv + i] = V::mk(zero, zero);
+            }
+            if (edge) {
+                const T2 v = p.v[j * nv + nr];
+                same = same && is_pzero(v.x) && is_pzero(v.y);
+                O.v[j * nv + nr] = V::mk(zero, zero);
+            }
+        }
+        if (UNI) speed_max = max_nonneg(speed_max, t_sqrt<T>(zero) + t_sqrt<T>(c2max));
+        unsigned long long b = (unsigned long long)__double_as_longlong(double(speed_max));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+        same = __all_sync(0xffffffffu, same);
+        if (lane == 0) {
+            O.rest_out[tile] = same ? 2 : 1;
+            O.rest_rate[tile] = b;
+        }
+        bits = max(bits, b);
+    }
     if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&p.scal->status, 2);
     __shared__ unsigned long long sh[kRestThreads / 32];
-    unsigned long long b = (unsigned long long)__double_as_longlong(double(speed_max));
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_down_sync(0xffffffffu, b, o));
-    if (lane == 0) sh[w] = b;
+    for (int o = 16; o > 0; o >>= 1) bits = max(bits, __shfl_down_sync(0xffffffffu, bits, o));
+    if (lane == 0) sh[w] = bits;
     __syncthreads();
     if (threadIdx.x == 0) {
-        for (int k = 1; k < kRestThreads / 32; ++k) b = max(b, sh[k]);
-        if (b != 0ull) atomicMax(&p.scal->maxbits, b);
+        for (int k = 1; k < kRestThreads / 32; ++k) bits = max(bits, sh[k]);
+        if (bits != 0ull) atomicMax(&p.scal->maxbits, bits);
     }
 }
 
@@ -1168,22 +1231,6 @@ struct RestCopyArgs {
     DevScalars* scal;
     double2* v;             // vertices of the copy written (the grid's last row and column)
 };
-
-// A tile is at rest when it and its eight neighbours (those inside the grid) took the
-// quiescent path in the step that wrote the copy read here.
-__device__ __forceinline__ bool tile_at_rest(const unsigned char* __restrict__ rest_in, int tile, int nbx, int nby)
-{
-    const int bx = tile % nbx, by = tile / nbx;
-    int rest = 1;
-#pragma unroll
-    for (int dy = -1; dy <= 1; ++dy)
-#pragma unroll
-        for (int dx = -1; dx <= 1; ++dx) {
-            const int tx = bx + dx, ty = by + dy;
-            if (tx >= 0 && tx < nbx && ty >= 0 && ty < nby) rest &= rest_in[ty * nbx + tx] != 0;
-        }
-    return rest != 0;
-}
 
 // One thread per tile: a tile at rest gets its flag for the next step (the copy kernel
 // moves its fields); every other tile is queued for the tile kernel, as the rest-tile
@@ -1402,9 +1449,25 @@ __global__ void __launch_bounds__(kThreads) k_courant_rates(const ParamsT<T> P, 
             const T2 fr = p.fr[m][c];
             if (pos(fr.x)) {
                 T pm, c2;
-                eos_eval<T>(P.mat[m], fr.y, Ic, pm, c2);
-                const T pmin = (T(1) - D) * P.mat[m].p_t * expansion_weight(P.mat[m], fr.y);
-                pm = pm < pmin ? pmin : pm;
+                // cold matter at its reference density (most of an impact grid before the
+                // shock): the Tillotson form's own values there are p = 0 and
+                // c^2 = A / rho0, which a warp of such cells takes without the form's two
+                // divisions (the FP64 pass over 4000 x 4000 cells was bound by the FP64
+                // pipe, 86 % busy, 2.03 ms)
+                const bool ref = same_bits(fr.y, P.mat[m].rho0) && is_pzero(p.I[c]) && P.mat[m].eos == SALEC_EOS_TILLOTSON;
+                if (!warp_any(!ref)) {
+                    pm = zero;
+                    c2 = P.mat[m].A * P.mat[m].inv_rho0;
+                    if (!(c2 > P.mat[m].c2_floor)) c2 = P.mat[m].c2_floor;
+                } else {
+                    eos_eval<T>(P.mat[m], fr.y, Ic, pm, c2);
+                }
+                if (nonzero(P.mat[m].p_t)) {
+                    const T pmin = (T(1) - D) * P.mat[m].p_t * expansion_weight(P.mat[m], fr.y);
+                    pm = pm < pmin ? pmin : pm;
+                } else if (pm < zero) {
+                    pm = zero;
+                }
                 phat += fr.x * pm;
                 phi += fr.x;
                 c2m = max_nonneg(c2m, c2);
@@ -1492,8 +1555,7 @@ struct Fused {
     }
     static cudaError_t rest(const ParamsT<T>& P, const OutPtrsT<T>& O, cudaStream_t s)
     {
-        constexpr int wpb = kRestThreads / 32;
-        k_rest_tiles<T, NM, STR, UNI, S::TW, S::TH><<<(tiles(P) + wpb - 1) / wpb, kRestThreads, 0, s>>>(P, O);
+        k_rest_tiles<T, NM, STR, UNI, S::TW, S::TH><<<(tiles(P) + kRestTiles - 1) / kRestTiles, kRestThreads, 0, s>>>(P, O);
         return cudaGetLastError();
     }
     static cudaError_t launch(const ParamsT<T>& P, const OutPtrsT<T>& O, cudaStream_t s)
@@ -1558,8 +1620,8 @@ cudaError_t launch_courant_rates(const ParamsT<T>& P, unsigned char* rest, cudaS
 }
 
 // One fused cycle: the Courant kernel (dt from the running maximum of the rates), the
-// rest-tile kernel (copies the tiles at rest, queues the others), the persistent tile
-// kernel.  With ev: an event before, one after the rest-tile kernel and one at the end.
+// rest-tile kernel (copies the tiles newly at rest, queues the moving ones), the persistent
+// tile kernel.  With ev: an event before, one after the rest-tile kernel and one at the end.
 template <typename T>
 cudaError_t launch_step_fused(const ParamsT<T>& P, const OutPtrsT<T>& O, cudaStream_t s, cudaEvent_t* ev)
 {

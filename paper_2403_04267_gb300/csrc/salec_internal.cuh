@@ -158,12 +158,14 @@ struct OutPtrsT {
     T* pr_psi2;
     T4* pr_v;
     T2* eosc;
-    // tiles at rest: rest_in[t] = 1 when the step that wrote the copy read here took tile t
-    // through the quiescent path (its outputs are then its inputs); this step writes
-    // rest_out.  work counts and hands out the tiles this step runs through the whole
+    // tiles at rest: rest_in[t] != 0 when the step that wrote the copy read here took tile t
+    // through the quiescent path (its outputs are then its inputs), 2 when the copy written
+    // here already holds the tile's values bit for bit and rest_rate[t] its Courant rate
+    // (FP64 bit pattern); this step writes rest_out.  work counts and hands out the tiles this step runs through the whole
     // cycle (list: their indices); work_next is zeroed for the next step.
     const unsigned char* rest_in;
     unsigned char* rest_out;
+    unsigned long long* rest_rate;
     TileWork* work;
     TileWork* work_next;
     int* list;
@@ -360,6 +362,8 @@ __device__ __forceinline__ bool is_nan(float x) { return (__float_as_int(x) & 0x
 __device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
 __device__ __forceinline__ bool is_pzero(double x) { return __double_as_longlong(x) == 0; }
 __device__ __forceinline__ bool is_pzero(float x) { return __float_as_int(x) == 0; }
+__device__ __forceinline__ bool same_bits(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_int(a) == __float_as_int(b); }
 __device__ __forceinline__ bool nonzero(float x) { return (__float_as_int(x) << 1) != 0; }
 // Any active lane of the warp: a warp-uniform branch condition.  Guarding FP64 work with it
 // keeps the compiler from turning a rarely taken branch into predicated instructions that
