@@ -58,13 +58,12 @@ long n_weights_bf16_t()
     return n;
 }
 
-// The backward pass reads its operands K-major (K = the batch for the weight gradients, K =
-// a layer's outputs for the activation gradients), so the TMA-fed GEMM serves it too: the
-// forward epilogues also write the activations transposed (HT, XT), the backward epilogues
-// the gradients transposed (GT), and the BF16 weights are kept transposed as well (wbfT).
+// The weight gradients contract over the batch: the training kernel leaves the activations
+// and the gradients of the pre-activations transposed (HT, XT, GT), and the BF16 weights are
+// kept transposed as well (wbfT) for the activation gradients.
 struct Layout {
-    size_t theta, m1, m2, grad, wmap, wbf, wmapT, wbfT, X, XT, Z[4], H[4], HT[4], Y, G[2], GT[2], part, loss, err,
-        ts, total;
+    size_t theta, m1, m2, grad, wmap, wbf, wmapT, wbfT, X, XT, HT[4], D, GT[kLayers], part[kLayers], loss, err, ts,
+        total;
     Layout(int bmax)
     {
         const long P = n_params(), W = n_weights_bf16(), WT = n_weights_bf16_t(), ldT = ld_t(bmax);
@@ -77,15 +76,12 @@ struct Layout {
         wbfT = take(WT * 2);
         X = take((size_t)bmax * kInLd * 2);
         XT = take((size_t)kInT * ldT * 2);
-        for (int l = 0; l < 4; ++l) Z[l] = take((size_t)bmax * kHid * 4);
-        for (int l = 0; l < 4; ++l) H[l] = take((size_t)bmax * kHid * 2);
         for (int l = 0; l < 4; ++l) HT[l] = take((size_t)kHidT * ldT * 2);
-        Y = take((size_t)bmax * SALEC_MLP_OUT * 4);
-        for (int l = 0; l < 2; ++l) G[l] = take((size_t)bmax * kHid * 2);
-        for (int l = 0; l < 2; ++l) GT[l] = take((size_t)kHid * ldT * 2);
-        part = take((size_t)kMaxSplit * kHid * (kHid + 1) * 4);   // split-K partials of a weight gradient
-        loss = take(8);
-        err = take(4);
+        D = take((size_t)SALEC_MLP_OUT * ldT * 4);
+        for (int l = 0; l < kLayers; ++l) GT[l] = take((size_t)kDims[l + 1] * ldT * 2);
+        for (int l = 0; l < kLayers; ++l) part[l] = take(dw_part_floats(l) * 4);   // split-K partials
+        loss = take(16);          // the sum of squared errors, then the error flag
+        err = loss + 8;
         ts = take(sizeof(TrainState));
         total = o;
     }
@@ -103,18 +99,10 @@ struct salec_mlp {
     int* wmapT = nullptr;
     __nv_bfloat16* wbfT = nullptr;
     __nv_bfloat16* X = nullptr;
-    __nv_bfloat16* XT = nullptr;
-    float* Z[4] = {};
-    __nv_bfloat16* H[4] = {};
-    __nv_bfloat16* HT[4] = {};
-    float* Y = nullptr;
-    __nv_bfloat16* G[2] = {};
-    __nv_bfloat16* GT[2] = {};
-    long ldT = 0;                         // row stride of the transposed buffers (batch_max, padded)
-    float* part = nullptr;
     double* loss = nullptr;
     int* errflag = nullptr;
     TrainState* ts = nullptr;
+    TrainNet net = {};                    // the arrays and TMA maps of the training kernels
     long steps = 0;                       // Adam steps taken
     // salec_mlp_train: a CUDA graph of kTrainChunk steps, for the arguments it was captured with
     cudaGraphExec_t tgraph = nullptr;
@@ -151,98 +139,6 @@ salec_status cuda_fail(salec_mlp* n, cudaError_t e, const char* where)
         if (e_ != cudaSuccess) return cuda_fail((n), e_, (where)); \
     } while (0)
 
-GemmArgs gemm0(int M, int N, int K, int* err)
-{
-    GemmArgs g = {};
-    g.M = M; g.N = N; g.K = K;
-    g.err = err;
-    return g;
-}
-
-// Forward layer l on X (already BF16): Z_l, H_l (and H_l^T) for the hidden layers; the
-// output layer with the plain store into y, or (with the targets t) the fused loss gradient.
-// The pre-activations and the transposed copies are kept only for a backward pass.
-GemmArgs fwd_gemm(salec_mlp* n, int l, int B, float* y, long ldy, const float* t, bool with_loss)
-{
-    const bool keep_z = with_loss;
-    const int ni = kDims[l], no = kDims[l + 1];
-    GemmArgs g = gemm0(B, no, ni, n->errflag);
-    g.A = l == 0 ? n->X : n->H[l - 1]; g.a_sm = l == 0 ? kInLd : kHid; g.a_sk = 1;
-    g.B = n->wbf + n->wbf_off[l]; g.b_sn = w_ld(l); g.b_sk = 1;
-    g.bias = n->theta + n->boff[l];
-    if (l + 1 < kLayers) {
-        g.epi = kEpiBiasGelu;
-        g.C = keep_z ? n->Z[l] : nullptr; g.ldc = kHid;
-        g.Hout = n->H[l]; g.ldh = kHid;
-        if (keep_z) { g.HoutT = n->HT[l]; g.ldhT = n->ldT; }
-    } else if (with_loss) {
-        g.epi = kEpiOutLoss;
-        g.C = y; g.ldc = ldy;
-        g.Tin = t; g.ldt = SALEC_MLP_OUT;
-        g.Hout = n->G[0]; g.ldh = kHid;
-        g.HoutT = n->GT[0]; g.ldhT = n->ldT;
-        g.grad_scale = 2.0f / ((float)B * (float)SALEC_MLP_OUT);
-        g.loss = n->loss;
-    } else {
-        g.epi = kEpiStore;
-        g.C = y; g.ldc = ldy;
-    }
-    return g;
-}
-
-// Backward, layer l, from G[cur] = dL/dZ_l (BF16, GT[cur] its transpose).
-// dW_l[o][i] = sum_b G[b][o] Hprev[b][i] and db_l[o] = sum_b G[b][o], as one product of
-// G^T (no x B) with [Hprev | 1]^T ((ni + 1) x B): the row of ones after the transposed
-// activations gives the bias gradient in the last column.
-GemmArgs dw_gemm(salec_mlp* n, int l, int B, int cur, float* grad)
-{
-    const int ni = kDims[l], no = kDims[l + 1];
-    GemmArgs g = gemm0(no, ni + 1, B, n->errflag);
-    g.A = n->GT[cur]; g.a_sm = n->ldT; g.a_sk = 1;
-    g.B = l > 0 ? n->HT[l - 1] : n->XT; g.b_sn = n->ldT; g.b_sk = 1;
-    g.epi = kEpiStore;
-    g.C = grad + n->woff[l]; g.ldc = ni;
-    g.Cb = grad + n->boff[l];
-    g.part = n->part;
-    return g;
-}
-
-// dL/dZ_{l-1}[b][i] = (sum_o G[b][o] W_l[o][i]) gelu'(Z_{l-1}[b][i]) into G[cur ^ 1] and its
-// transpose, W_l^T K-major (l >= 1).
-GemmArgs dh_gemm(salec_mlp* n, int l, int B, int cur)
-{
-    const int ni = kDims[l], no = kDims[l + 1];
-    GemmArgs g = gemm0(B, ni, no, n->errflag);
-    g.A = n->G[cur]; g.a_sm = kHid; g.a_sk = 1;
-    g.B = n->wbfT + n->wbfT_off[l]; g.b_sn = wt_ld(l); g.b_sk = 1;
-    g.epi = kEpiGeluBwd;
-    g.Zin = n->Z[l - 1]; g.ldz = kHid;
-    g.Hout = n->G[cur ^ 1]; g.ldh = kHid;
-    g.HoutT = n->GT[cur ^ 1]; g.ldhT = n->ldT;
-    return g;
-}
-
-salec_status forward_impl(salec_mlp* n, int B, float* y, long ldy, const float* t, bool with_loss)
-{
-    for (int l = 0; l < kLayers; ++l)
-        MLP_CUDA(n, launch_gemm(fwd_gemm(n, l, B, y, ldy, t, with_loss), n->stream), "mlp forward gemm");
-    return SALEC_OK;
-}
-
-// backward pass from G[0] = dL/dY: weight and bias gradients into grad.  Every operand is
-// read K-major, so every GEMM is TMA-fed.
-salec_status backward_impl(salec_mlp* n, int B, float* grad)
-{
-    int cur = 0;
-    for (int l = kLayers - 1; l >= 0; --l) {
-        MLP_CUDA(n, launch_gemm(dw_gemm(n, l, B, cur, grad), n->stream), "mlp weight-gradient gemm");
-        if (l == 0) break;
-        MLP_CUDA(n, launch_gemm(dh_gemm(n, l, B, cur), n->stream), "mlp activation-gradient gemm");
-        cur ^= 1;
-    }
-    return SALEC_OK;
-}
-
 salec_status check_batch(salec_mlp* n, int B)
 {
     if (!n) return SALEC_EINVAL;
@@ -252,20 +148,31 @@ salec_status check_batch(salec_mlp* n, int B)
 
 constexpr int kTrainChunk = 25;
 
+// the inputs as BF16 rows of 8 and transposed, for a training pass
+cudaError_t inputs(salec_mlp* n, const float* x_dev, int B, cudaStream_t s)
+{
+    return launch_inputs_bf16(x_dev, B, SALEC_MLP_IN, kInLd, n->X, s, n->net.p.XT, n->net.p.ldT);
+}
+
+TrainLaunch train_launch(int B, const float* t_dev, const float* lr_dev, float beta1, float beta2, float eps)
+{
+    TrainLaunch t = {};
+    t.B = B;
+    t.t = t_dev;
+    t.lr = lr_dev;
+    t.adam.beta1 = beta1; t.adam.beta2 = beta2; t.adam.eps = eps;
+    t.adam.table = lr_dev != nullptr;
+    return t;
+}
+
 // One step of a multi-step call: its learning rate and bias corrections from the device
 // state, then the gradient and the Adam update (the inputs are already in X).
 salec_status train_one(salec_mlp* n, int B, const float* t_dev, const float* lr_dev, float beta1, float beta2,
                        float eps)
 {
-    MLP_CUDA(n, launch_train_begin(n->ts, lr_dev, beta1, beta2, n->loss, n->stream), "mlp train step");
-    salec_status st = forward_impl(n, B, n->Y, SALEC_MLP_OUT, t_dev, true);
-    if (st != SALEC_OK) return st;
-    st = backward_impl(n, B, n->grad);
-    if (st != SALEC_OK) return st;
-    AdamArgs a;
-    a.lr = 0.0f; a.c1 = 0.0f; a.c2 = 0.0f;
-    a.beta1 = beta1; a.beta2 = beta2; a.eps = eps; a.ts = n->ts;
-    MLP_CUDA(n, launch_adam(n->theta, n->m1, n->m2, n->grad, n_params(), a, n->wmap, n->wbf, n->stream, n->wmapT, n->wbfT), "mlp adam");
+    TrainNet* net = &n->net;
+    MLP_CUDA(n, launch_train_pass(&net, 1, train_launch(B, t_dev, lr_dev, beta1, beta2, eps), nullptr, n->stream),
+             "mlp train step");
     return SALEC_OK;
 }
 
@@ -339,37 +246,15 @@ salec_status gfail(salec_mlp_group* g, salec_status st, const std::string& msg)
         if (e_ != cudaSuccess) return gfail((g), SALEC_ECUDA, std::string(where) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
-// One training step of every member: the step's start, the forward pass, the backward pass
-// and Adam, each GEMM one launch for all members (the inputs are already in each X, X^T).
+// One training step of every member, each kernel one launch for all members (the inputs are
+// already in each X, X^T).
 salec_status group_train_one(salec_mlp_group* G, cudaStream_t s, int B, const float* t_dev, const float* lr_dev,
                              float beta1, float beta2, float eps)
 {
+    TrainNet* nets[kMaxGroup];
     const int n = (int)G->nets.size();
-    GemmArgs args[kMaxGroup];
-    BeginGroup bg;
-    for (int k = 0; k < n; ++k) { bg.ts[k] = G->nets[k]->ts; bg.loss[k] = G->nets[k]->loss; }
-    GROUP_CUDA(G, launch_train_begin_group(bg, n, lr_dev, beta1, beta2, s), "group train step");
-    for (int l = 0; l < kLayers; ++l) {
-        for (int k = 0; k < n; ++k) args[k] = fwd_gemm(G->nets[k], l, B, G->nets[k]->Y, SALEC_MLP_OUT, t_dev, true);
-        GROUP_CUDA(G, launch_gemm_group(args, n, s), "group forward gemm");
-    }
-    int cur = 0;
-    for (int l = kLayers - 1; l >= 0; --l) {
-        for (int k = 0; k < n; ++k) args[k] = dw_gemm(G->nets[k], l, B, cur, G->nets[k]->grad);
-        GROUP_CUDA(G, launch_gemm_group(args, n, s), "group weight-gradient gemm");
-        if (l == 0) break;
-        for (int k = 0; k < n; ++k) args[k] = dh_gemm(G->nets[k], l, B, cur);
-        GROUP_CUDA(G, launch_gemm_group(args, n, s), "group activation-gradient gemm");
-        cur ^= 1;
-    }
-    AdamGroup ag;
-    for (int k = 0; k < n; ++k) {
-        salec_mlp* m = G->nets[k];
-        ag.theta[k] = m->theta; ag.m1[k] = m->m1; ag.m2[k] = m->m2; ag.grad[k] = m->grad;
-        ag.wbf[k] = m->wbf; ag.wbfT[k] = m->wbfT; ag.ts[k] = m->ts;
-    }
-    GROUP_CUDA(G, launch_adam_group(ag, n, n_params(), beta1, beta2, eps, G->nets[0]->wmap, G->nets[0]->wmapT, s),
-               "group adam");
+    for (int k = 0; k < n; ++k) nets[k] = &G->nets[k]->net;
+    GROUP_CUDA(G, launch_train_pass(nets, n, train_launch(B, t_dev, lr_dev, beta1, beta2, eps), nullptr, s), "group train step");
     return SALEC_OK;
 }
 
@@ -440,19 +325,6 @@ salec_status salec_mlp_create(int batch_max, void* dev_buf, size_t bytes, void* 
     n->wmapT = reinterpret_cast<int*>(b + L.wmapT);
     n->wbfT = reinterpret_cast<__nv_bfloat16*>(b + L.wbfT);
     n->X = reinterpret_cast<__nv_bfloat16*>(b + L.X);
-    n->XT = reinterpret_cast<__nv_bfloat16*>(b + L.XT);
-    n->ldT = ld_t(batch_max);
-    for (int l = 0; l < 4; ++l) {
-        n->Z[l] = reinterpret_cast<float*>(b + L.Z[l]);
-        n->H[l] = reinterpret_cast<__nv_bfloat16*>(b + L.H[l]);
-        n->HT[l] = reinterpret_cast<__nv_bfloat16*>(b + L.HT[l]);
-    }
-    n->Y = reinterpret_cast<float*>(b + L.Y);
-    for (int l = 0; l < 2; ++l) {
-        n->G[l] = reinterpret_cast<__nv_bfloat16*>(b + L.G[l]);
-        n->GT[l] = reinterpret_cast<__nv_bfloat16*>(b + L.GT[l]);
-    }
-    n->part = reinterpret_cast<float*>(b + L.part);
     n->loss = reinterpret_cast<double*>(b + L.loss);
     n->errflag = reinterpret_cast<int*>(b + L.err);
     n->ts = reinterpret_cast<TrainState*>(b + L.ts);
@@ -476,17 +348,33 @@ salec_status salec_mlp_create(int batch_max, void* dev_buf, size_t bytes, void* 
         n->boff[l] = o;
         o += no;
     }
+    NetPtrs& p = n->net.p;
+    p.X = n->X;
+    p.W1 = n->wbf;
+    for (int l = 0; l < kLayers; ++l) {
+        p.bias[l] = n->theta + n->boff[l];
+        p.GT[l] = reinterpret_cast<__nv_bfloat16*>(b + L.GT[l]);
+        p.part[l] = reinterpret_cast<float*>(b + L.part[l]);
+    }
+    p.XT = reinterpret_cast<__nv_bfloat16*>(b + L.XT);
+    for (int l = 0; l < 4; ++l) p.HT[l] = reinterpret_cast<__nv_bfloat16*>(b + L.HT[l]);
+    p.ldT = ld_t(batch_max);
+    p.D = reinterpret_cast<float*>(b + L.D);
+    p.theta = n->theta; p.m1 = n->m1; p.m2 = n->m2;
+    p.wbf = n->wbf; p.wbfT = n->wbfT;
+    p.ts = n->ts; p.loss = n->loss; p.err = n->errflag;
     // the rows of ones under the transposed activations (BF16 1.0 = 0x3f80): columns past
     // the batch lie outside the tensor map and read as zero
-    std::vector<uint16_t> ones((size_t)n->ldT, 0x3f80u);
+    std::vector<uint16_t> ones((size_t)p.ldT, 0x3f80u);
     cudaError_t e = cudaMemsetAsync(dev_buf, 0, L.total, n->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(n->wmap, wmap.data(), P * sizeof(int), cudaMemcpyHostToDevice, n->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(n->wmapT, wmapT.data(), P * sizeof(int), cudaMemcpyHostToDevice, n->stream);
     for (int l = 0; l < 4 && e == cudaSuccess; ++l)
-        e = cudaMemcpyAsync(n->HT[l] + (long)kHid * n->ldT, ones.data(), ones.size() * 2, cudaMemcpyHostToDevice, n->stream);
+        e = cudaMemcpyAsync(p.HT[l] + (long)kHid * p.ldT, ones.data(), ones.size() * 2, cudaMemcpyHostToDevice, n->stream);
     if (e == cudaSuccess)
-        e = cudaMemcpyAsync(n->XT + (long)SALEC_MLP_IN * n->ldT, ones.data(), ones.size() * 2, cudaMemcpyHostToDevice,
+        e = cudaMemcpyAsync(p.XT + (long)SALEC_MLP_IN * p.ldT, ones.data(), ones.size() * 2, cudaMemcpyHostToDevice,
                             n->stream);
+    if (e == cudaSuccess) e = make_weight_maps(&n->net);
     if (e == cudaSuccess) e = cudaStreamSynchronize(n->stream);
     if (e != cudaSuccess) {
         delete n;
@@ -523,16 +411,15 @@ salec_status salec_mlp_forward(salec_mlp* n, const float* x_dev, int batch, floa
     salec_status st = check_batch(n, batch);
     if (st != SALEC_OK) return st;
     if (!x_dev || !y_dev) return fail(n, SALEC_EINVAL, "null pointer");
+    bool done = false;
+    MLP_CUDA(n, launch_infer_small(n->net, x_dev, batch, y_dev, n->stream, &done), "mlp forward");
+    if (done) return SALEC_OK;
     MLP_CUDA(n, launch_inputs_bf16(x_dev, batch, SALEC_MLP_IN, kInLd, n->X, n->stream), "mlp input");
-    // all five layers in one kernel, activations on chip; the layer-by-layer GEMMs when
-    // the weights cannot be addressed by TMA
     FusedLaunch f;
     f.B = batch; f.X = n->X; f.ld_x = kInLd; f.Y = y_dev; f.err = n->errflag;
     for (int l = 0; l < kLayers; ++l) { f.W[l] = n->wbf + n->wbf_off[l]; f.bias[l] = n->theta + n->boff[l]; }
-    const cudaError_t e = launch_mlp_forward_fused(f, n->stream);
-    if (e == cudaSuccess) return SALEC_OK;
-    if (e != cudaErrorNotSupported) return cuda_fail(n, e, "mlp fused forward");
-    return forward_impl(n, batch, y_dev, SALEC_MLP_OUT, nullptr, false);
+    MLP_CUDA(n, launch_mlp_forward_fused(f, n->stream), "mlp forward");
+    return SALEC_OK;
 }
 
 salec_status salec_mlp_gradient(salec_mlp* n, const float* x_dev, const float* t_dev, int batch, float* grad_dev,
@@ -543,18 +430,16 @@ salec_status salec_mlp_gradient(salec_mlp* n, const float* x_dev, const float* t
     if (st != SALEC_OK) return st;
     if (!x_dev || !t_dev) return fail(n, SALEC_EINVAL, "null pointer");
     float* grad = grad_dev ? grad_dev : n->grad;
-    MLP_CUDA(n, cudaMemsetAsync(n->loss, 0, 8, n->stream), "mlp loss reset");
-    MLP_CUDA(n, launch_inputs_bf16(x_dev, batch, SALEC_MLP_IN, kInLd, n->X, n->stream, n->XT, n->ldT), "mlp input");
-    st = forward_impl(n, batch, n->Y, SALEC_MLP_OUT, t_dev, true);
-    if (st != SALEC_OK) return st;
-    st = backward_impl(n, batch, grad);
-    if (st != SALEC_OK) return st;
+    MLP_CUDA(n, inputs(n, x_dev, batch, n->stream), "mlp input");
+    TrainNet* net = &n->net;
+    MLP_CUDA(n, launch_train_pass(&net, 1, train_launch(batch, t_dev, nullptr, 0.0f, 0.0f, 0.0f), grad, n->stream),
+             "mlp gradient");
     if (loss_host) {
-        double s = 0.0;
-        MLP_CUDA(n, cudaMemcpyAsync(&s, n->loss, 8, cudaMemcpyDeviceToHost, n->stream), "mlp loss read");
+        struct { double sse; int err, pad; } r;
+        MLP_CUDA(n, cudaMemcpyAsync(&r, n->loss, sizeof(r), cudaMemcpyDeviceToHost, n->stream), "mlp loss read");
         MLP_CUDA(n, cudaStreamSynchronize(n->stream), "mlp loss sync");
-        *loss_host = s / ((double)batch * SALEC_MLP_OUT);
-        return salec_mlp_check(n);
+        *loss_host = r.sse / ((double)batch * SALEC_MLP_OUT);
+        if (r.err) return fail(n, SALEC_ECUDA, "a tensor-core wait ran out of time");
     }
     return SALEC_OK;
 }
@@ -568,18 +453,14 @@ salec_status salec_mlp_train_step(salec_mlp* n, const float* x_dev, const float*
     if (!x_dev || !t_dev) return fail(n, SALEC_EINVAL, "null pointer");
     if (!(lr >= 0.0f) || !(beta1 >= 0.0f && beta1 < 1.0f) || !(beta2 >= 0.0f && beta2 < 1.0f) || !(eps > 0.0f))
         return fail(n, SALEC_EINVAL, "bad Adam hyper-parameters");
-    MLP_CUDA(n, cudaMemsetAsync(n->loss, 0, 8, n->stream), "mlp loss reset");
-    MLP_CUDA(n, launch_inputs_bf16(x_dev, batch, SALEC_MLP_IN, kInLd, n->X, n->stream, n->XT, n->ldT), "mlp input");
-    st = forward_impl(n, batch, n->Y, SALEC_MLP_OUT, t_dev, true);
-    if (st != SALEC_OK) return st;
-    st = backward_impl(n, batch, n->grad);
-    if (st != SALEC_OK) return st;
+    MLP_CUDA(n, inputs(n, x_dev, batch, n->stream), "mlp input");
     n->steps += 1;
-    AdamArgs a;
-    a.lr = lr; a.beta1 = beta1; a.beta2 = beta2; a.eps = eps; a.ts = nullptr;
-    a.c1 = (float)(1.0 / (1.0 - std::pow((double)beta1, (double)n->steps)));
-    a.c2 = (float)(1.0 / (1.0 - std::pow((double)beta2, (double)n->steps)));
-    MLP_CUDA(n, launch_adam(n->theta, n->m1, n->m2, n->grad, n_params(), a, n->wmap, n->wbf, n->stream, n->wmapT, n->wbfT), "mlp adam");
+    TrainLaunch t = train_launch(batch, t_dev, nullptr, beta1, beta2, eps);
+    t.adam.lr = lr;
+    t.adam.c1 = (float)(1.0 / (1.0 - std::pow((double)beta1, (double)n->steps)));
+    t.adam.c2 = (float)(1.0 / (1.0 - std::pow((double)beta2, (double)n->steps)));
+    TrainNet* net = &n->net;
+    MLP_CUDA(n, launch_train_pass(&net, 1, t, nullptr, n->stream), "mlp train step");
     if (sse_dev) MLP_CUDA(n, cudaMemcpyAsync(sse_dev, n->loss, 8, cudaMemcpyDeviceToDevice, n->stream), "mlp loss copy");
     return SALEC_OK;
 }
@@ -596,7 +477,7 @@ salec_status salec_mlp_train(salec_mlp* n, const float* x_dev, const float* t_de
     if (!(beta1 >= 0.0f && beta1 < 1.0f) || !(beta2 >= 0.0f && beta2 < 1.0f) || !(eps > 0.0f))
         return fail(n, SALEC_EINVAL, "bad Adam hyper-parameters");
     if (n->steps + (long)steps > 0x7fffffffL) return fail(n, SALEC_EINVAL, "step count overflow");
-    MLP_CUDA(n, launch_inputs_bf16(x_dev, batch, SALEC_MLP_IN, kInLd, n->X, n->stream, n->XT, n->ldT), "mlp input");
+    MLP_CUDA(n, inputs(n, x_dev, batch, n->stream), "mlp input");
     MLP_CUDA(n, launch_train_reset(n->ts, (int)n->steps, n->stream), "mlp train reset");
     // the first step with plain launches (it also sets the kernels' attributes), then whole
     // chunks as graph replays, then the rest
@@ -637,10 +518,10 @@ salec_status salec_gemm_bf16(int M, int N, int K, const void* A, long a_sm, long
 {
     if (M < 0 || N < 0 || K < 0) return SALEC_EINVAL;
     if (M > 0 && N > 0 && (!C || (K > 0 && (!A || !B)))) return SALEC_EINVAL;   // K = 0: C = 0, A and B unused
-    GemmArgs g = gemm0(M, N, K, nullptr);
+    GemmArgs g = {};
+    g.M = M; g.N = N; g.K = K;
     g.A = static_cast<const __nv_bfloat16*>(A); g.a_sm = a_sm; g.a_sk = a_sk;
     g.B = static_cast<const __nv_bfloat16*>(B); g.b_sn = b_sn; g.b_sk = b_sk;
-    g.epi = kEpiStore;
     g.C = C; g.ldc = ldc;
     if (launch_gemm(g, static_cast<cudaStream_t>(stream)) != cudaSuccess) return SALEC_ECUDA;
     return SALEC_OK;
@@ -679,7 +560,7 @@ salec_status salec_mlp_train_group(salec_mlp_group* G, const float* x_dev, const
     }
     cudaStream_t s = G->stream;
     for (salec_mlp* m : G->nets) {
-        GROUP_CUDA(G, launch_inputs_bf16(x_dev, batch, SALEC_MLP_IN, kInLd, m->X, s, m->XT, m->ldT), "group input");
+        GROUP_CUDA(G, inputs(m, x_dev, batch, s), "group input");
         GROUP_CUDA(G, launch_train_reset(m->ts, (int)m->steps, s), "group train reset");
     }
     // the first step with plain launches (it also sets the kernels' attributes), then whole
