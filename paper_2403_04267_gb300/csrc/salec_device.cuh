@@ -94,6 +94,56 @@ struct Geo {
     }
 };
 
+// The Courant rate (|v| + c) / L of a cell only counts where it raises the running maximum,
+// and in the FP64 form its two square roots and four vertex speeds are a third of phase 0's
+// work on the FP64 pipe.  An upper bound in FP32 (from the high words, integer
+// instructions) decides first: warps none of whose cells can exceed the maximum seen so far
+// skip the FP64 evaluation.  The maximum that results is the same.
+__device__ __forceinline__ float up_f32(double x)       // >= |x|; +inf for NaN and beyond FP32
+{
+    const int h = __double2hiint(x) & 0x7fffffff;
+    if (h < 0x38200000) return 1.2e-38f;
+    if (h >= 0x47e00000) return __int_as_float(0x7f800000);
+    return __int_as_float(((h - 0x38000000) << 3) + 16);
+}
+__device__ __forceinline__ float down_f32(double x)     // <= x for x >= 0
+{
+    const int h = __double2hiint(x);
+    if (h < 0x38200000) return 0.0f;
+    if (h >= 0x47e00000) return 3.0e38f;
+    return __int_as_float((h - 0x38000000) << 3);
+}
+__device__ __forceinline__ float up_w(double2 v)
+{
+    const float x = up_f32(v.x), y = up_f32(v.y);
+    return __fmaf_ru(x, x, __fmul_ru(y, y));
+}
+__device__ __forceinline__ float up_w(float2) { return 0.0f; }
+// whether (|v| + c) / L of a cell with squared sound speed c2 and corner velocities va.. vd may
+// exceed `run` (the mixed form always evaluates: its square roots are cheap)
+template <typename T, typename T2>
+__device__ __forceinline__ bool rate_may_raise(T2 va, T2 vb, T2 vc, T2 vd, T c2, T ilen, bool scaled, double run)
+{
+    if (sizeof(T) == 4) return true;
+    const float w = fmaxf(fmaxf(up_w(va), up_w(vb)), fmaxf(up_w(vc), up_w(vd)));
+    float r = __fadd_ru(__fsqrt_ru(w), __fsqrt_ru(up_f32(double(c2))));
+    if (scaled) r = __fmul_ru(r, up_f32(double(ilen)));
+    return !(r <= down_f32(run));
+}
+
+// a / b with y = 1 / b (within an ulp): the quotient corrected by its exact remainder
+// (Markstein, IBM J. Res. Dev. 34, 1990), three instructions on the FP64 pipe instead of a
+// division's ten; exactly 1 for a == b
+__device__ __forceinline__ double div_by(double a, double b, double y)
+{
+    const double q = a * y;
+    return __fma_rn(__fma_rn(-q, b, a), y, q);
+}
+__device__ __forceinline__ float div_by(float a, float b, float) { return a / b; }
+
+__device__ __forceinline__ bool finite_pos(double x) { return __double_as_longlong(x) > 0 && __double2hiint(x) < 0x7ff00000; }
+__device__ __forceinline__ bool finite_pos(float x) { return __float_as_int(x) > 0 && __float_as_int(x) < 0x7f800000; }
+
 // What a dual face carries: mass f, momentum f w and kinetic energy f |w|^2 / 2 with the
 // upwind vertex velocity w.
 template <typename T>

@@ -344,11 +344,15 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
             const T uL = half * (va.x + vd.x), uR = half * (vb.x + vc.x);
             const T uB = half * (va.y + vb.y), uT = half * (vd.y + vc.y);
             const T div = (GE::flux_r(P, i, j, uL, uR) + p.A_Z[i] * (uT - uB)) * GE::ivol(P, i, j);
-            const T cs = t_sqrt<T>(c2m);
-            const T iphi = NM == 1 ? one : one / phi;
+            constexpr bool F64 = sizeof(T) == 8;      // (as phase 0 of the phase kernels)
+            T iphi = one;
+            if (NM > 1 && (!F64 || warp_any(phi != one))) iphi = one / phi;
             pbar = NM == 1 ? p1 : phat * iphi;
+            T cs = zero;
+            if (!F64) cs = t_sqrt<T>(c2m);
             T q = zero;
-            if (neg(div)) {
+            if (F64 ? warp_any(neg(div)) && neg(div) : neg(div)) {
+                if (F64) cs = t_sqrt<T>(c2m);
                 const T rb = NM == 1 ? r1 : mass * iphi;
                 const T Lc = GE::len(P, i, j);
                 q = rb * (P.cq * (UNI ? P.dx2 : Lc * Lc) * div * div - P.cl * Lc * cs * div);
@@ -380,6 +384,7 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
         const int v = j * nv + i;
         T Pc[4] = {zero, zero, zero, zero}, Pp[4] = {zero, zero, zero, zero};
         T devr_rad = zero, devz_rad = zero, devr_ver = zero, devz_ver = zero, mass = zero;
+        const bool strip = j < P.pb || i > nr - P.pr;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const int ci = (q == 0 || q == 3) ? i - 1 : i;
@@ -389,7 +394,8 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
             const T2 pm = s_PM[kc];
             Pc[q] = pm.x;
             mass += T(0.25) * pm.y;
-            if (STR || P.pr > 0 || P.pb > 0) {
+            // (without strength only the strips need the pressure's deviation)
+            if (STR || warp_any(strip)) {
                 T phi;
                 if (PBPHI) {
                     phi = s_pbphi[kc].y;
@@ -557,19 +563,29 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
         for (int m = 0; m < NM; ++m) {
             const T2 fr = s_fro[m][kc];
             if (pos(fr.x)) {
-                const T Vm = fr.x * Vc;
-                const T VmL = NM == 1 ? Vm + dVmat : Vm + fr.x / phi * dVmat;
-                bad |= !pos(VmL) || !pos(fr.y);     // non-positive Lagrangian volume or density
-                // unchanged volume: V_m / V_m^L is exactly 1 (no division)
-                s_frL[m][kc] = V::mk(VmL / VLc, warp_any(nonzero(dV)) ? fr.y * (Vm / VmL) : fr.y);
+                // a cell full of one material: one division instead of three (as phase 2 of
+                // the phase kernels)
+                const bool whole = sizeof(T) == 8 && same_bits(fr.x, one) && same_bits(phi, one) && finite_pos(VLc);
+                if (sizeof(T) == 8 && !warp_any(!whole)) {
+                    bad |= !pos(fr.y);
+                    s_frL[m][kc] = V::mk(one, warp_any(nonzero(dV)) ? fr.y * (Vc / VLc) : fr.y);
+                } else {
+                    const T Vm = fr.x * Vc;
+                    const T VmL = NM == 1 ? Vm + dVmat : Vm + fr.x / phi * dVmat;
+                    bad |= !pos(VmL) || !pos(fr.y);     // non-positive Lagrangian volume or density
+                    // unchanged volume: V_m / V_m^L is exactly 1 (no division)
+                    s_frL[m][kc] = V::mk(VmL / VLc, warp_any(nonzero(dV)) ? fr.y * (Vm / VmL) : fr.y);
+                }
                 if (STR && P.mat[m].strength == SALEC_STRENGTH_COLLINS) {
                     const MatT<T>& mm = P.mat[m];
                     const T pb = s_pbphi[kc].x;
                     G += fr.x * mm.G;
                     Y += fr.x * yield_eval<T>(mm, pb, D, T(Ic), fr.y);
-                    T ef = mm.B_dam * (pb - mm.p_bd);
-                    ef = ef < mm.eps_fb ? mm.eps_fb : ef;
-                    iepsf += fr.x / ef;
+                    if (sizeof(T) == 4) {
+                        T ef = mm.B_dam * (pb - mm.p_bd);
+                        ef = ef < mm.eps_fb ? mm.eps_fb : ef;
+                        iepsf += fr.x / ef;
+                    }
                 }
             } else {
                 s_frL[m][kc] = V::mk(zero, zero);
@@ -577,8 +593,9 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
         }
         if (bad) atomicOr(&p.scal->status, 1);
         if (STR) {
-            const T iphi = one / phi;
-            G *= iphi; Y *= iphi; iepsf *= iphi;
+            T iphi = one;
+            if (sizeof(T) == 4 || warp_any(phi != one)) iphi = one / phi;
+            G *= iphi; Y *= iphi;
             if (pos(G)) {
                 const T omega = half * (dvr_dz - dvz_dr);
                 const T erz = half * (dvr_dz + dvz_dr);
@@ -590,6 +607,18 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
                 const T ntt = -(nrr + nzz);
                 const T J2 = half * (nrr * nrr + nzz * nzz + ntt * ntt) + nrz * nrz;
                 if (J2 > Y * Y) {
+                    // FP64 form: the failure strain only where the matter yields
+#pragma unroll
+                    for (int m = 0; m < NM; ++m) {
+                        if (sizeof(T) == 4) break;
+                        const MatT<T>& mm = P.mat[m];
+                        const T fm = s_fro[m][kc].x;
+                        if (!pos(fm) || mm.strength != SALEC_STRENGTH_COLLINS) continue;
+                        T ef = mm.B_dam * (s_pbphi[kc].x - mm.p_bd);
+                        ef = ef < mm.eps_fb ? mm.eps_fb : ef;
+                        iepsf += fm / ef;
+                    }
+                    iepsf *= iphi;
                     const T sq = t_sqrt<T>(J2);
                     const T kq = Y / sq;
                     nrr *= kq; nzz *= kq; nrz *= kq;
@@ -725,7 +754,7 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
             T Mkeep = zero, Vkeep = zero, fnew[NM];
 #pragma unroll
             for (int m = 0; m < NM; ++m) {
-                fnew[m] = Vm[m] / Vc;
+                fnew[m] = div_by(Vm[m], Vc, GE::ivol(P, i, j));
                 if (fnew[m] < P.f_min) {
                     const bool tally = own && nonzero(Mm[m]);
                     if (warp_any(tally) && tally) t_disc += double(Mm[m]);
@@ -910,6 +939,7 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
     __syncthreads();
 
     // ---- phase 3c: heat to the own cells; the Courant rate of the new state (Eq. 14)
+    const double run = sizeof(T) == 8 ? __longlong_as_double((long long)*(volatile const unsigned long long*)&p.scal->maxbits) : 0.0;
     for (int k = tid; k < TW * TH; k += NT) {
         const int lx = H + k % TW, ly = H + k / TW, i = x0 + lx, j = y0 + ly;
         if (i >= nr || j >= nz) continue;
@@ -966,15 +996,26 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
         const T c2m = ec.y;
         if (pos(phi)) {
             const T2 va = s_vn[ka], vb = s_vn[ka + 1], vc = s_vn[ka + VW + 1], vd = s_vn[ka + VW];
-            T w = va.x * va.x + va.y * va.y;
-            w = max_nonneg(w, vb.x * vb.x + vb.y * vb.y);
-            w = max_nonneg(w, vc.x * vc.x + vc.y * vc.y);
-            w = max_nonneg(w, vd.x * vd.x + vd.y * vd.y);
-            T speed = t_sqrt<T>(w) + t_sqrt<T>(c2m);
-            if (!UNI) speed = speed * GE::ilen(P, i, j);
-            if (is_nan(speed)) atomicOr(&p.scal->status, 2);
-            speed_max = max_nonneg(speed_max, speed);
+            const bool raise = rate_may_raise<T>(va, vb, vc, vd, c2m, UNI ? one : GE::ilen(P, i, j), !UNI,
+                                                 max_nonneg(run, double(speed_max)));
+            if (sizeof(T) == 4 || (warp_any(raise) && raise)) {
+                T w = va.x * va.x + va.y * va.y;
+                w = max_nonneg(w, vb.x * vb.x + vb.y * vb.y);
+                w = max_nonneg(w, vc.x * vc.x + vc.y * vc.y);
+                w = max_nonneg(w, vd.x * vd.x + vd.y * vd.y);
+                T speed = t_sqrt<T>(w) + t_sqrt<T>(c2m);
+                if (!UNI) speed = speed * GE::ilen(P, i, j);
+                if (is_nan(speed)) atomicOr(&p.scal->status, 2);
+                speed_max = max_nonneg(speed_max, speed);
+            }
         }
+    }
+    // FP64 form: a warp that raised the maximum says so now, for the tests of later tiles
+    if (sizeof(T) == 8 && __any_sync(0xffffffffu, double(speed_max) > run)) {
+        unsigned long long b = (unsigned long long)__double_as_longlong(double(speed_max));
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
+        if ((tid & 31) == 0) atomicMax(&p.scal->maxbits, b);
     }
 
     }   // not quiescent
@@ -1441,7 +1482,8 @@ __global__ void __launch_bounds__(kThreads) k_courant_rates(const ParamsT<T> P, 
     bool q = true;          // cells outside the grid read as empty: quiescent
     if (i < nr && j < P.nz) {
         const int c = j * nr + i;
-        T phi = zero, c2m = zero, phat = zero, p1 = zero;
+        T phi = zero, c2m = zero, phat = zero, p1 = zero, c_ref = zero;
+        bool all_ref = true;
         const T Ic = T(p.I[c]);
         const T D = STR ? p.s2d[c].y : zero;
 #pragma unroll
@@ -1451,16 +1493,17 @@ __global__ void __launch_bounds__(kThreads) k_courant_rates(const ParamsT<T> P, 
                 T pm, c2;
                 // cold matter at its reference density (most of an impact grid before the
                 // shock): the Tillotson form's own values there are p = 0 and
-                // c^2 = A / rho0, which a warp of such cells takes without the form's two
-                // divisions (the FP64 pass over 4000 x 4000 cells was bound by the FP64
-                // pipe, 86 % busy, 2.03 ms)
+                // c^2 = A / rho0, which a warp of such cells takes from the material constants
+                // (with the square root that its rate needs) instead of forming them: the FP64
+                // pass over 4000 x 4000 cells was bound by the FP64 pipe (86 % busy, 2.03 ms)
                 const bool ref = same_bits(fr.y, P.mat[m].rho0) && is_pzero(p.I[c]) && P.mat[m].eos == SALEC_EOS_TILLOTSON;
                 if (!warp_any(!ref)) {
                     pm = zero;
-                    c2 = P.mat[m].A * P.mat[m].inv_rho0;
-                    if (!(c2 > P.mat[m].c2_floor)) c2 = P.mat[m].c2_floor;
+                    c2 = P.mat[m].c2_ref;
+                    c_ref = max_nonneg(c_ref, P.mat[m].c_ref);
                 } else {
                     eos_eval<T>(P.mat[m], fr.y, Ic, pm, c2);
+                    all_ref = false;
                 }
                 if (nonzero(P.mat[m].p_t)) {
                     const T pmin = (T(1) - D) * P.mat[m].p_t * expansion_weight(P.mat[m], fr.y);
@@ -1479,7 +1522,17 @@ __global__ void __launch_bounds__(kThreads) k_courant_rates(const ParamsT<T> P, 
         const int nv = nr + 1;
         const T2 va = p.v[j * nv + i], vb = p.v[j * nv + i + 1];
         const T2 vc = p.v[(j + 1) * nv + i + 1], vd = p.v[(j + 1) * nv + i];
-        if (pos(phi)) {
+        const double run = sizeof(T) == 8 ? __longlong_as_double((long long)*(volatile const unsigned long long*)&p.scal->maxbits) : 0.0;
+        const bool still = all_ref && !nonzero(va.x) && !nonzero(va.y) && !nonzero(vb.x) && !nonzero(vb.y) &&
+                           !nonzero(vc.x) && !nonzero(vc.y) && !nonzero(vd.x) && !nonzero(vd.y);
+        const bool raise = pos(phi) && rate_may_raise<T>(va, vb, vc, vd, c2m, UNI ? T(1) : GE::ilen(P, i, j), !UNI, run);
+        if (!warp_any(raise && !still)) {
+            // at rest: sqrt(0) + c
+            if (raise) {
+                speed = c_ref;
+                if (!UNI) speed = speed * GE::ilen(P, i, j);
+            }
+        } else if (raise) {
             T w = va.x * va.x + va.y * va.y;
             w = max_nonneg(w, vb.x * vb.x + vb.y * vb.y);
             w = max_nonneg(w, vc.x * vc.x + vc.y * vc.y);

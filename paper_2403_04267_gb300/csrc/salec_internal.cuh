@@ -11,6 +11,7 @@
 
 #include <cuda.h>
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -52,6 +53,7 @@ struct MatT {
     int eos, strength;
     T rho0, inv_rho0, rho0sq_E0, A, B, E0, a, b, alpha, beta, Eiv, Ecv, inv_dE, gamma;
     T Yi0, mui, Yim, Yd0, mud, Ydm, inv_Yspan, G, eps_fb, B_dam, p_bd, p_t, c2_floor;
+    T c2_ref, c_ref;        // Tillotson: c^2 and c of cold matter at rho0 (where p = 0)
     T rho_f, inv_rho_f;     // the Tillotson density floor 1e-12 rho0 and its reciprocal
 };
 typedef MatT<double> Mat;
@@ -202,6 +204,9 @@ inline MatT<T> to_mat(const salec_material& s)
     m.G = T(s.strength == SALEC_STRENGTH_COLLINS ? s.G : 0.0);
     m.eps_fb = T(s.eps_fb); m.B_dam = T(s.B_dam); m.p_bd = T(s.p_bd); m.p_t = T(s.p_t);
     m.c2_floor = T(s.eos == SALEC_EOS_TILLOTSON ? 0.01 * s.A / s.rho0 : 0.0);
+    m.c2_ref = m.A * m.inv_rho0;
+    if (!(m.c2_ref > m.c2_floor)) m.c2_ref = m.c2_floor;
+    m.c_ref = T(sqrt(m.c2_ref));
     m.rho_f = T(1e-12 * s.rho0); m.inv_rho_f = T(1.0 / (1e-12 * s.rho0));
     return m;
 }
@@ -220,6 +225,34 @@ template <> __host__ __device__ inline float t_sqrt<float>(float x) { return sqr
 // before the tension cut-off and c^2 = dp/drho + p/rho^2 dp/dI of the branch (in the
 // blend, the blend of the two branches' values), floored.
 // ---------------------------------------------------------------------------------
+// Sign tests on the bit pattern: integer instructions instead of floating-point compares
+// (FP64 compares issue on the FP64 pipe, the bottleneck of the FP64 form).  pos(x): x > 0
+// (or +NaN); neg(x): x < 0 (or -NaN), -0 excluded: a resting face (velocity -0)
+// moves nothing and costs nothing.
+__device__ __forceinline__ bool pos(double x) { return __double_as_longlong(x) > 0; }
+__device__ __forceinline__ bool neg(double x)
+{
+    const long long b = __double_as_longlong(x);
+    return b < 0 && (b << 1) != 0;
+}
+__device__ __forceinline__ bool pos(float x) { return __float_as_int(x) > 0; }
+__device__ __forceinline__ bool neg(float x)
+{
+    const int b = __float_as_int(x);
+    return b < 0 && (b << 1) != 0;
+}
+__device__ __forceinline__ bool is_nan(double x)
+{
+    return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
+}
+__device__ __forceinline__ bool is_nan(float x) { return (__float_as_int(x) & 0x7fffffff) > 0x7f800000; }
+// x != 0 (either sign of zero counts as zero) on the bit pattern
+__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
+__device__ __forceinline__ bool is_pzero(double x) { return __double_as_longlong(x) == 0; }
+__device__ __forceinline__ bool is_pzero(float x) { return __float_as_int(x) == 0; }
+__device__ __forceinline__ bool same_bits(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
+__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_int(a) == __float_as_int(b); }
+__device__ __forceinline__ bool nonzero(float x) { return (__float_as_int(x) << 1) != 0; }
 // a < b for b > 0 on the bit patterns: an integer compare (any negative a, and -0, is below)
 __device__ __forceinline__ bool below_bits(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
 __device__ __forceinline__ bool below_bits(float a, float b) { return __float_as_int(a) < __float_as_int(b); }
@@ -229,7 +262,14 @@ template <typename T>
 __host__ __device__ __forceinline__ void eos_eval(const MatT<T>& m, T rho_in, T I_in, T& p_out, T& c2_out)
 {
     const T zero = T(0), one = T(1), two = T(2);
+#ifdef __CUDA_ARCH__
+    // FP64 form: the tests on the bit patterns, in integer instructions (a NaN as the
+    // comparisons take it); the mixed form has no register to spare for them
+    constexpr bool F64 = sizeof(T) == 8;
+    const T I = (F64 ? pos(I_in) && !is_nan(I_in) : I_in > zero) ? I_in : zero;
+#else
     const T I = I_in > zero ? I_in : zero;
+#endif
     if (m.eos == SALEC_EOS_IDEAL_GAS) {
         const T gm1 = m.gamma - one;
         p_out = gm1 * rho_in * I;
@@ -240,13 +280,29 @@ __host__ __device__ __forceinline__ void eos_eval(const MatT<T>& m, T rho_in, T 
     // c^2 no longer depends on rho and p is proportional to it (p = a rho I once the
     // exponential terms vanish), so below rho_f the pressure is scaled back by rho / rho_f;
     // the rho^-2 terms below stay finite in FP32
+#ifdef __CUDA_ARCH__
+    const T rho = (F64 ? !below_bits(rho_in, m.rho_f) && !is_nan(rho_in) : rho_in > m.rho_f) ? rho_in : m.rho_f;
+#else
     const T rho = rho_in > m.rho_f ? rho_in : m.rho_f;
-    // two divisions: 1/rho and 1/w0 (1/(E0 eta^2) = (rho0^2/E0) / rho^2)
-    const T irho = one / rho;
+#endif
     const T mu = (rho - m.rho0) * m.inv_rho0;
-    const T ie = m.rho0sq_E0 * irho * irho;            // 1 / (E0 eta^2)
-    const T w0 = I * ie + one;
-    const T iw = one / w0;
+    // 1/rho, and 1/w0 with w0 = I / (E0 eta^2) + 1, 1/(E0 eta^2) = (rho0^2/E0) / rho^2.  The FP64
+    // form takes both from one division, of which each costs ten instructions of its bound
+    // pipe: with q = rho^2 w0, 1/rho = q / (rho q) and 1/w0 = rho^2 / q
+    T irho, ie, iw;
+    if (sizeof(T) == 8) {
+        const T rho2 = rho * rho;
+        const T q = I * m.rho0sq_E0 + rho2;
+        const T r = one / (rho * q);
+        irho = q * r;
+        ie = m.rho0sq_E0 * irho * irho;                // 1 / (E0 eta^2)
+        iw = rho2 * (rho * r);
+    } else {
+        irho = one / rho;
+        ie = m.rho0sq_E0 * irho * irho;
+        const T w0 = I * ie + one;
+        iw = one / w0;
+    }
     const T bw = m.b * iw;                             // b / w0
     const T dw = bw * iw * I * ie;                     // b I / (w0^2 E0 eta^2)
     // compressed branch and its partial derivatives
@@ -255,7 +311,11 @@ __host__ __device__ __forceinline__ void eos_eval(const MatT<T>& m, T rho_in, T 
     const T pc_I = rho * (m.a + bw - dw);
     const T irho2 = irho * irho;
     T p, c2;
+#ifdef __CUDA_ARCH__
+    if ((F64 ? !below_bits(rho, m.rho0) : rho >= m.rho0) || I <= m.Eiv) {
+#else
     if (rho >= m.rho0 || I <= m.Eiv) {
+#endif
         p = pc;
         c2 = pc_r + pc * irho2 * pc_I;
     } else {
@@ -294,7 +354,11 @@ __host__ __device__ __forceinline__ void eos_eval(const MatT<T>& m, T rho_in, T 
 #else
     if (rho_in < m.rho_f) p *= (rho_in > zero ? rho_in : zero) * m.inv_rho_f;
 #endif
+#ifdef __CUDA_ARCH__
+    if (F64 ? !below_bits(m.c2_floor, c2) || is_nan(c2) : !(c2 > m.c2_floor)) c2 = m.c2_floor;     // the floor is positive
+#else
     if (!(c2 > m.c2_floor)) c2 = m.c2_floor;
+#endif
     p_out = p;
     c2_out = c2;
 }
@@ -331,40 +395,19 @@ __host__ __device__ __forceinline__ T yield_eval(const MatT<T>& m, T p_in, T D, 
     T Y = (one - D) * Yi + D * Yd;
     if (I > zero) {
         if (!(I < m.Eiv)) return zero;
+#ifdef __CUDA_ARCH__
+        // FP64 form: tanh is exactly 1 from an argument of 19.1 on, so a warp of cold rock (most
+        // of a target) needs neither it nor its division
+        const bool warm = sizeof(T) == 4 || !(T(17) * I < m.Eiv);
+        if (sizeof(T) == 4 || (warp_any(warm) && warm)) Y *= t_tanh<T>(T(1.2) * (m.Eiv / I - one));
+#else
         Y *= t_tanh<T>(T(1.2) * (m.Eiv / I - one));
+#endif
     }
     Y *= expansion_weight(m, rho);
     return Y > zero ? Y : zero;
 }
 
-// Sign tests on the bit pattern: integer instructions instead of floating-point compares
-// (FP64 compares issue on the FP64 pipe, the bottleneck of the FP64 form).  pos(x): x > 0
-// (or +NaN); neg(x): x < 0 (or -NaN), -0 excluded: a resting face (velocity -0)
-// moves nothing and costs nothing.
-__device__ __forceinline__ bool pos(double x) { return __double_as_longlong(x) > 0; }
-__device__ __forceinline__ bool neg(double x)
-{
-    const long long b = __double_as_longlong(x);
-    return b < 0 && (b << 1) != 0;
-}
-__device__ __forceinline__ bool pos(float x) { return __float_as_int(x) > 0; }
-__device__ __forceinline__ bool neg(float x)
-{
-    const int b = __float_as_int(x);
-    return b < 0 && (b << 1) != 0;
-}
-__device__ __forceinline__ bool is_nan(double x)
-{
-    return (__double_as_longlong(x) & 0x7fffffffffffffffLL) > 0x7ff0000000000000LL;
-}
-__device__ __forceinline__ bool is_nan(float x) { return (__float_as_int(x) & 0x7fffffff) > 0x7f800000; }
-// x != 0 (either sign of zero counts as zero) on the bit pattern
-__device__ __forceinline__ bool nonzero(double x) { return (__double_as_longlong(x) << 1) != 0; }
-__device__ __forceinline__ bool is_pzero(double x) { return __double_as_longlong(x) == 0; }
-__device__ __forceinline__ bool is_pzero(float x) { return __float_as_int(x) == 0; }
-__device__ __forceinline__ bool same_bits(double a, double b) { return __double_as_longlong(a) == __double_as_longlong(b); }
-__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_int(a) == __float_as_int(b); }
-__device__ __forceinline__ bool nonzero(float x) { return (__float_as_int(x) << 1) != 0; }
 // Any active lane of the warp: a warp-uniform branch condition.  Guarding FP64 work with it
 // keeps the compiler from turning a rarely taken branch into predicated instructions that
 // every warp would issue (FP64 instructions occupy the FP64 pipe even when predicated off);

@@ -46,6 +46,8 @@ __device__ __forceinline__ void body_phase0(const ParamsT<T>& P, int bx, int by,
     // uniform grid takes the max of |v| + c and divides dx by it).  The max is exact in T,
     // so it is taken in T and the block's value converted to FP64 once.
     T speed = zero;
+    // the maximum so far (a later, larger one only makes the test below skip less)
+    const double run = sizeof(T) == 8 ? __longlong_as_double((long long)*(volatile const unsigned long long*)&p.scal->maxbits) : 0.0;
     if (i < nr && j < P.nz) {
         const int c = j * nr + i;
         T phat = zero, phi = zero, mass = zero, c2m = zero, p1 = zero, r1 = zero;
@@ -75,12 +77,19 @@ __device__ __forceinline__ void body_phase0(const ParamsT<T>& P, int bx, int by,
             const T uL = half * (va.x + vd.x), uR = half * (vb.x + vc.x);
             const T uB = half * (va.y + vb.y), uT = half * (vd.y + vc.y);
             const T div = (GE::flux_r(P, i, j, uL, uR) + p.A_Z[i] * (uT - uB)) * GE::ivol(P, i, j);
-            const T cs = t_sqrt<T>(c2m);
-            // one material: p_bar = p and rho_bar = rho; otherwise divide by Phi once
-            const T iphi = NM == 1 ? one : one / phi;
+            // one material: p_bar = p and rho_bar = rho; otherwise divide by Phi once.  The FP64
+            // form skips the division in warps of full cells (Phi exactly 1) and the sound
+            // speed where nothing is compressed; the mixed form, bound by latency at an
+            // occupancy its registers set, is faster without the tests (139 against 173 us)
+            constexpr bool F64 = sizeof(T) == 8;
+            T iphi = one;
+            if (NM > 1 && (!F64 || warp_any(phi != one))) iphi = one / phi;
             pbar = NM == 1 ? p1 : phat * iphi;
+            T cs = zero;
+            if (!F64) cs = t_sqrt<T>(c2m);
             T q = zero;
-            if (neg(div)) {
+            if (F64 ? warp_any(neg(div)) && neg(div) : neg(div)) {
+                if (F64) cs = t_sqrt<T>(c2m);
                 const T rb = NM == 1 ? r1 : mass * iphi;
                 const T L = GE::len(P, i, j);
                 q = rb * (P.cq * (UNI ? P.dx2 : L * L) * div * div - P.cl * L * cs * div);
@@ -88,13 +97,16 @@ __device__ __forceinline__ void body_phase0(const ParamsT<T>& P, int bx, int by,
             Pc = phat + phi * q;
             const T over = pbar - p.p0[j];
             if (over > p.pmax[c]) p.pmax[c] = over;
-            T w = va.x * va.x + va.y * va.y;
-            w = max_nonneg(w, vb.x * vb.x + vb.y * vb.y);
-            w = max_nonneg(w, vc.x * vc.x + vc.y * vc.y);
-            w = max_nonneg(w, vd.x * vd.x + vd.y * vd.y);
-            speed = t_sqrt<T>(w) + cs;
-            if (!UNI) speed = speed * GE::ilen(P, i, j);
-            if (is_nan(speed)) atomicOr(&p.scal->status, 2);
+            const bool raise = rate_may_raise<T>(va, vb, vc, vd, c2m, UNI ? one : GE::ilen(P, i, j), !UNI, run);
+            if (!F64 || (warp_any(raise) && raise)) {
+                T w = va.x * va.x + va.y * va.y;
+                w = max_nonneg(w, vb.x * vb.x + vb.y * vb.y);
+                w = max_nonneg(w, vc.x * vc.x + vc.y * vc.y);
+                w = max_nonneg(w, vd.x * vd.x + vd.y * vd.y);
+                speed = t_sqrt<T>(w) + (F64 ? t_sqrt<T>(c2m) : cs);
+                if (!UNI) speed = speed * GE::ilen(P, i, j);
+                if (is_nan(speed)) atomicOr(&p.scal->status, 2);
+            }
         }
         p.PM[c] = V::mk(Pc, mass * GE::vol(P, i, j));
         p.pbphi[c] = V::mk(pbar, phi);
@@ -154,6 +166,56 @@ __device__ __forceinline__ void body_phase1(const ParamsT<T>& P, int bx, int by,
     const int v = j * (nr + 1) + i;
     T Pc[4] = {zero, zero, zero, zero}, Pp[4] = {zero, zero, zero, zero};
     T devr_rad = zero, devz_rad = zero, devr_ver = zero, devz_ver = zero, mass = zero;
+    const bool strip = j < P.pb || i > nr - P.pr;
+    if (sizeof(T) == 8 && UNI) {
+        // FP64 form on a uniform grid: the corner terms of the two cells of a column share
+        // their geometry factors, so the stresses are added (or subtracted) first and scaled
+        // once; full cells (Phi exactly 1) need no product with Phi, and the pressure's
+        // deviation from its reference only counts in the strips
+        T Srr[4] = {zero, zero, zero, zero}, Szz[4] = {zero, zero, zero, zero}, Srz[4] = {zero, zero, zero, zero};
+        T phi[4] = {one, one, one, one};
+        bool part = false;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const int ci = (k == 0 || k == 3) ? i - 1 : i;
+            const int cj = (k < 2) ? j - 1 : j;
+            if (ci < 0 || ci >= nr || cj < 0 || cj >= nz) continue;
+            const int c = cj * nr + ci;
+            const typename V::T2 pm = p.PM[c];
+            Pc[k] = pm.x;
+            mass += pm.y;
+            if (STR || P.pr > 0 || P.pb > 0) phi[k] = p.pbphi[c].y;
+            if (STR) {
+                const typename V::T2 s01 = p.s01[c];
+                Srr[k] = s01.x; Szz[k] = s01.y; Srz[k] = p.s2d[c].x;
+                part = part || !same_bits(phi[k], one);
+            }
+        }
+        mass *= T(0.25);
+        if (warp_any(strip)) {
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int ci = (k == 0 || k == 3) ? i - 1 : i;
+                const int cj = (k < 2) ? j - 1 : j;
+                if (strip && ci >= 0 && ci < nr && cj >= 0 && cj < nz) Pp[k] = Pc[k] - phi[k] * p.p0[cj];
+            }
+        }
+        if (STR) {
+            if (warp_any(part)) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    Srr[k] *= phi[k]; Szz[k] *= phi[k]; Srz[k] *= phi[k];
+                }
+            }
+            const T hl = i > 0 ? half * p.A_Z[i - 1] : zero, hr = i < nr ? half * p.A_Z[i] : zero;
+            const T rr_r = Srr[1] + Srr[2], rr_l = Srr[0] + Srr[3];
+            const T zz = (Szz[0] + Szz[3]) + (Szz[1] + Szz[2]);
+            devr_rad = hr * rr_r - hl * rr_l + GE::quarter_v_rc(P, 0, 0) * ((rr_r + rr_l) + zz);
+            devz_rad = hr * (Srz[1] + Srz[2]) - hl * (Srz[0] + Srz[3]);
+            devr_ver = hr * (Srz[2] - Srz[1]) + hl * (Srz[3] - Srz[0]);
+            devz_ver = hr * (Szz[2] - Szz[1]) + hl * (Szz[3] - Szz[0]);
+        }
+    } else
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int ci = (k == 0 || k == 3) ? i - 1 : i;
@@ -287,6 +349,7 @@ __device__ __forceinline__ void body_phase2(const ParamsT<T>& P, int bx, int by,
     const T Pc = pm.x, M = pm.y;
     T work = zero, Pi_rad = -Pc * rad_flux, Pi_ver = -Pc * ver_flux;
     T dvr_dz = zero, dvz_dr = zero, srr = zero, szz = zero, srz = zero, D = zero;
+    const bool strip = j < P.pb || i >= nr - P.pr;
     if (STR) {
         const typename V::T2 s01 = p.s01[c], s2d = p.s2d[c];
         srr = s01.x; szz = s01.y; srz = s2d.x; D = s2d.y;
@@ -295,8 +358,10 @@ __device__ __forceinline__ void body_phase2(const ParamsT<T>& P, int bx, int by,
         const T Srr = phi * srr, Szz = phi * szz, Srz = phi * srz, Stt = -(Srr + Szz);
         const T erz = half * (dvr_dz + dvz_dr);
         work = dt * Vc * (Srr * err + Szz * ezz + Stt * ett + two * Srz * erz);
-        Pi_rad += Vc * (Srr * err + Stt * ett + Srz * dvz_dr);
-        Pi_ver += Vc * (Szz * ezz + Srz * dvr_dz);
+        if (sizeof(T) == 4 || (warp_any(strip) && strip)) {
+            Pi_rad += Vc * (Srr * err + Stt * ett + Srz * dvz_dr);
+            Pi_ver += Vc * (Szz * ezz + Srz * dvr_dz);
+        }
     }
     T psi2 = zero;
     if (j < P.pb) {
@@ -331,20 +396,32 @@ __device__ __forceinline__ void body_phase2(const ParamsT<T>& P, int bx, int by,
     for (int m = 0; m < NM; ++m) {
         const typename V::T2 fr = p.fr[m][c];
         if (pos(fr.x)) {
-            const T Vm = fr.x * Vc;
-            // one material: f_m / Phi = 1; true divisions keep a resting cell exact
-            const T VmL = NM == 1 ? Vm + dVmat : Vm + fr.x / phi * dVmat;
-            bad |= !pos(VmL) || !pos(fr.y);     // non-positive Lagrangian volume or density
-            // unchanged volume: V_m / V_m^L is exactly 1 (no division)
-            p.frL[m][c] = V::mk(VmL / VLc, warp_any(nonzero(dV)) ? fr.y * (Vm / VmL) : fr.y);
+            // a cell full of one material (f_m and Phi exactly 1): V_m = V, V_m^L = V^L and
+            // f_m^L = 1 as the divisions below would give them, so in the FP64 form a warp of
+            // such cells, most of a target, takes one division instead of three (phase 2 172 ->
+            // 135 us on 800 x 800 cells with the skips below; the mixed form gains nothing)
+            const bool whole = sizeof(T) == 8 && same_bits(fr.x, one) && same_bits(phi, one) && finite_pos(VLc);
+            if (sizeof(T) == 8 && !warp_any(!whole)) {
+                bad |= !pos(fr.y);
+                p.frL[m][c] = V::mk(one, warp_any(nonzero(dV)) ? fr.y * (Vc / VLc) : fr.y);
+            } else {
+                const T Vm = fr.x * Vc;
+                // one material: f_m / Phi = 1; true divisions keep a resting cell exact
+                const T VmL = NM == 1 ? Vm + dVmat : Vm + fr.x / phi * dVmat;
+                bad |= !pos(VmL) || !pos(fr.y);     // non-positive Lagrangian volume or density
+                // unchanged volume: V_m / V_m^L is exactly 1 (no division)
+                p.frL[m][c] = V::mk(VmL / VLc, warp_any(nonzero(dV)) ? fr.y * (Vm / VmL) : fr.y);
+            }
             if (STR && P.mat[m].strength == SALEC_STRENGTH_COLLINS) {
                 const MatT<T>& mm = P.mat[m];
                 const T pb = p.pbphi[c].x;
                 G += fr.x * mm.G;
                 Y += fr.x * yield_eval<T>(mm, pb, D, T(Ic), fr.y);
-                T ef = mm.B_dam * (pb - mm.p_bd);
-                ef = ef < mm.eps_fb ? mm.eps_fb : ef;
-                iepsf += fr.x / ef;
+                if (sizeof(T) == 4) {
+                    T ef = mm.B_dam * (pb - mm.p_bd);
+                    ef = ef < mm.eps_fb ? mm.eps_fb : ef;
+                    iepsf += fr.x / ef;
+                }
             }
         } else {
             p.frL[m][c] = V::mk(zero, zero);
@@ -352,8 +429,9 @@ __device__ __forceinline__ void body_phase2(const ParamsT<T>& P, int bx, int by,
     }
     if (bad) atomicOr(&p.scal->status, 1);
     if (STR) {
-        const T iphi = one / phi;
-        G *= iphi; Y *= iphi; iepsf *= iphi;
+        T iphi = one;
+        if (sizeof(T) == 4 || warp_any(phi != one)) iphi = one / phi;
+        G *= iphi; Y *= iphi;
         if (pos(G)) {
             const T omega = half * (dvr_dz - dvz_dr);
             const T erz = half * (dvr_dz + dvz_dr);
@@ -365,6 +443,18 @@ __device__ __forceinline__ void body_phase2(const ParamsT<T>& P, int bx, int by,
             const T ntt = -(nrr + nzz);
             const T J2 = half * (nrr * nrr + nzz * nzz + ntt * ntt) + nrz * nrz;
             if (J2 > Y * Y) {
+                // FP64 form: the failure strain only where the matter yields
+#pragma unroll
+                for (int m = 0; m < NM; ++m) {
+                    if (sizeof(T) == 4) break;
+                    const MatT<T>& mm = P.mat[m];
+                    const T fm = p.fr[m][c].x;
+                    if (!pos(fm) || mm.strength != SALEC_STRENGTH_COLLINS) continue;
+                    T ef = mm.B_dam * (p.pbphi[c].x - mm.p_bd);
+                    ef = ef < mm.eps_fb ? mm.eps_fb : ef;
+                    iepsf += fm / ef;
+                }
+                iepsf *= iphi;
                 const T sq = t_sqrt<T>(J2);
                 const T k = Y / sq;
                 nrr *= k; nzz *= k; nrz *= k;
@@ -404,18 +494,25 @@ __device__ __forceinline__ T vertical_dV(const ParamsT<T>& P, int i, int j, T dt
     return dt * P.p.A_Z[i] * u;
 }
 
+// The FP64 form with several materials skips, warp by warp, the materials that no cell of the
+// warp or neighbour of one holds (phase 3a 212 -> 166 us on 800 x 800 cells, with the quotient
+// by the cell volume); in the mixed form the test's registers cost more occupancy than the
+// skipped work saves (253 against 270 us).
+template <typename T, int NM> struct ByMat { static constexpr bool value = sizeof(T) == 8 && NM > 1; };
+
 // Flux of |dV| of the donor cell's Lagrangian contents, added with sign sgn to acc.
 // Returns the moved mass and energy (energy for the PML auxiliaries only); an inflow
 // (sgn > 0) adds (I_donor - I_self) * mass to the energy change.
 template <typename T, int NM, bool STR>
 __device__ __forceinline__ void move(const ParamsT<T>& P, int donor, T adV, T sgn, double Iself, bool strip,
-                                     Acc<T, NM>& acc, T& mass_out, T& e_out)
+                                     unsigned use, Acc<T, NM>& acc, T& mass_out, T& e_out)
 {
     typedef VT<T> V;
     const PtrsT<T>& p = P.p;
     T vmat = T(0), mass = T(0);
 #pragma unroll
     for (int m = 0; m < NM; ++m) {
+        if (ByMat<T, NM>::value && !(use >> m & 1u)) continue;
         const typename V::T2 fl = p.frL[m][donor];
         const T dv = adV * fl.x;
         const T dm = fl.y * dv;
@@ -462,21 +559,33 @@ __device__ __forceinline__ void body_phase3a(const ParamsT<T>& P, int bx, int by
         const bool strip = j < P.pb || i >= nr - P.pr;
         T FRm = zero, FRe = zero, FZm = zero, FZe = zero;
         T fm, fe;
+        // materials that some cell of the warp, or a neighbour of one, holds; the others
+        // contribute zeros to every sum below
+        unsigned use = 0u;
+        if (ByMat<T, NM>::value) {
+            const int cl = i > 0 ? c - 1 : c, cr = i + 1 < nr ? c + 1 : c, cb = j > 0 ? c - nr : c, ct = j + 1 < nz ? c + nr : c;
+#pragma unroll
+            for (int m = 0; m < NM; ++m) {
+                const typename V::T2* f = p.frL[m];
+                const bool any = nonzero(f[c].x) || nonzero(f[cl].x) || nonzero(f[cr].x) || nonzero(f[cb].x) || nonzero(f[ct].x);
+                if (warp_any(any)) use |= 1u << m;
+            }
+        }
         // left face r_i: positive dV flows from (i-1,j) into this cell
         {
             const T dV = radial_dV<T, UNI>(P, i, j, dt);
             T sm = zero;
             if (!warp_any(nonzero(dV))) {
-            } else if (pos(dV)) { move<T, NM, STR>(P, c - 1, dV, one, ILc, strip, acc, fm, fe); sm = fm; FRm -= fm; FRe -= fe; }
-            else if (neg(dV)) { move<T, NM, STR>(P, c, -dV, -one, ILc, strip, acc, fm, fe); sm = -fm; FRm += fm; FRe += fe; }
+            } else if (pos(dV)) { move<T, NM, STR>(P, c - 1, dV, one, ILc, strip, use, acc, fm, fe); sm = fm; FRm -= fm; FRe -= fe; }
+            else if (neg(dV)) { move<T, NM, STR>(P, c, -dV, -one, ILc, strip, use, acc, fm, fe); sm = -fm; FRm += fm; FRe += fe; }
             p.dMR[j * (nr + 1) + i] = sm;
         }
         // right face r_{i+1}
         {
             const T dV = radial_dV<T, UNI>(P, i + 1, j, dt);
             if (!warp_any(nonzero(dV))) {
-            } else if (pos(dV)) { move<T, NM, STR>(P, c, dV, -one, ILc, strip, acc, fm, fe); FRm += fm; FRe += fe; }
-            else if (neg(dV)) { move<T, NM, STR>(P, c + 1, -dV, one, ILc, strip, acc, fm, fe); FRm -= fm; FRe -= fe; }
+            } else if (pos(dV)) { move<T, NM, STR>(P, c, dV, -one, ILc, strip, use, acc, fm, fe); FRm += fm; FRe += fe; }
+            else if (neg(dV)) { move<T, NM, STR>(P, c + 1, -dV, one, ILc, strip, use, acc, fm, fe); FRm -= fm; FRe -= fe; }
             if (i == nr - 1) p.dMR[j * (nr + 1) + nr] = zero;
         }
         // bottom face z_j
@@ -484,8 +593,8 @@ __device__ __forceinline__ void body_phase3a(const ParamsT<T>& P, int bx, int by
             const T dV = vertical_dV<T>(P, i, j, dt);
             T sm = zero;
             if (!warp_any(nonzero(dV))) {
-            } else if (pos(dV)) { move<T, NM, STR>(P, c - nr, dV, one, ILc, strip, acc, fm, fe); sm = fm; FZm -= fm; FZe -= fe; }
-            else if (neg(dV)) { move<T, NM, STR>(P, c, -dV, -one, ILc, strip, acc, fm, fe); sm = -fm; FZm += fm; FZe += fe; }
+            } else if (pos(dV)) { move<T, NM, STR>(P, c - nr, dV, one, ILc, strip, use, acc, fm, fe); sm = fm; FZm -= fm; FZe -= fe; }
+            else if (neg(dV)) { move<T, NM, STR>(P, c, -dV, -one, ILc, strip, use, acc, fm, fe); sm = -fm; FZm += fm; FZe += fe; }
             p.dMZ[j * nr + i] = sm;
         }
         // top face z_{j+1}: above the domain only outflow (inflow is void)
@@ -494,11 +603,11 @@ __device__ __forceinline__ void body_phase3a(const ParamsT<T>& P, int bx, int by
             T sm = zero;
             if (!warp_any(nonzero(dV))) {
             } else if (pos(dV)) {
-                move<T, NM, STR>(P, c, dV, -one, ILc, strip, acc, fm, fe);
+                move<T, NM, STR>(P, c, dV, -one, ILc, strip, use, acc, fm, fe);
                 FZm += fm; FZe += fe; sm = fm;
                 if (j == nz - 1) t_out += double(fm);
             } else if (neg(dV) && j + 1 < nz) {
-                move<T, NM, STR>(P, c + nr, -dV, one, ILc, strip, acc, fm, fe); FZm -= fm; FZe -= fe;
+                move<T, NM, STR>(P, c + nr, -dV, one, ILc, strip, use, acc, fm, fe); FZm -= fm; FZe -= fe;
             }
             if (j == nz - 1) p.dMZ[nz * nr + i] = sm;
         }
@@ -510,6 +619,10 @@ __device__ __forceinline__ void body_phase3a(const ParamsT<T>& P, int bx, int by
         T MLtot = zero, VLmat = zero, dMtot = zero, dVtot = zero;
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
+            if (ByMat<T, NM>::value && !(use >> m & 1u)) {
+                Vm[m] = Mm[m] = rn[m] = zero;
+                continue;
+            }
             const typename V::T2 fl = p.frL[m][c];
             const T VmL = fl.x * VLc;
             const T MmL = fl.y * VmL;
@@ -537,7 +650,10 @@ __device__ __forceinline__ void body_phase3a(const ParamsT<T>& P, int bx, int by
         T Mkeep = zero, Vkeep = zero, fnew[NM];
 #pragma unroll
         for (int m = 0; m < NM; ++m) {
-            fnew[m] = Vm[m] / Vc;    // a true division: exact 1 for a full resting cell
+            fnew[m] = zero;
+            if (ByMat<T, NM>::value && !(use >> m & 1u)) continue;
+            // the rounded quotient: exact 1 for a full resting cell
+            fnew[m] = div_by(Vm[m], Vc, Geo<T, UNI>::ivol(P, i, j));
             if (fnew[m] < P.f_min) {
                 if (warp_any(nonzero(Mm[m])) && nonzero(Mm[m])) t_disc += double(Mm[m]);
                 Vm[m] = zero;
@@ -779,6 +895,7 @@ __device__ __forceinline__ void body_phase3b(const ParamsT<T>& P, int bx, int by
                 const int ci = (k == 0 || k == 3) ? i - 1 : i;
                 const int cj = (k < 2) ? j - 1 : j;
                 if (ci < 0 || ci >= nr || cj < 0 || cj >= nz) continue;
+                if (!warp_any(!occupied)) break;
                 for (int mm = 0; mm < P.nmat; ++mm) occupied |= pos(p.fr[mm][cj * nr + ci].x);
             }
             if (occupied) {
