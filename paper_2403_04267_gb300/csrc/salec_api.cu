@@ -26,7 +26,10 @@ constexpr size_t kAlign = 256;
 // partials.
 const dim3 kShapes[] = {dim3(32, 4), dim3(32, 8), dim3(32, 16), dim3(64, 4), dim3(64, 8), dim3(128, 2), dim3(128, 4)};
 constexpr int kNumShapes = sizeof(kShapes) / sizeof(kShapes[0]);
-const dim3 kDefaultShape(32, 8);
+// (the autotuner's choice for most kernels: 800 x 800 FP64 588 -> 572 us per step against 32 x 8
+// blocks, the mixed layered grid 63 -> 61, 100 x 100 FP64, whose 52 blocks of 256 would use a
+// third of the SMs, 52 -> 38)
+const dim3 kDefaultShape(32, 4);
 
 // Offsets of every array inside the state buffer.  The persistent part (scalars, tables,
 // fields, PML auxiliaries) comes first so a checkpoint is one contiguous range.
@@ -783,14 +786,18 @@ salec_status salec_finalize(salec_ctx* ctx)
     if (e != cudaSuccess) return cuda_check(ctx, e, "fused step set-up");
     for (int k = 0; k < 2; ++k) ctx->Od[k].ctas = ctx->Of[k].ctas = ctas;
     if (!mixed(ctx)) prepare_beside(ctx);
-    // Default form.  Without gravity the fused form: its quiescent tiles (matter at rest
-    // at zero pressure) only read and write their state, which on an impact grid is most of
-    // it (4000 x 4000: mixed form 0.41 against 0.90 ms per step, FP64 1.26 against 7.16; a
-    // 1600 x 1600 grid with a fifth of its vertices moving: 0.125 against 0.172, 1.02
-    // against 1.47).  Under gravity no tile is quiescent (a loaded column is not at zero
-    // pressure) and the phase kernels, which compute no cell twice, are faster (the
-    // paper's layered grid: 0.054 against 0.087 ms, FP64 0.45 against 0.70).
-    ctx->form = g.gravity == 0.0 ? SALEC_STEP_FUSED : SALEC_STEP_PHASES;
+    // Default form.  Without gravity, on grids beyond a size, the fused form: its tiles at
+    // rest (matter at rest at zero pressure, most of a large impact grid) cost next to
+    // nothing (4000 x 4000: mixed form 0.08 against 0.90 ms per step, FP64 0.29 against
+    // 7.1).  Under gravity no tile is quiescent (a loaded column is not at zero pressure) and
+    // the phase kernels, which compute no cell twice, are faster (the paper's layered grid:
+    // 0.054 against 0.087 ms, FP64 0.45 against 0.70).  So they are on small grids, whose few
+    // tiles leave most SMs idle while one SM works through a tile's frame: FP64 100 x 100
+    // 58 against 103 us per step, 250 x 250 72 against 94, 400 x 400 (half at rest) 119
+    // against 90; mixed 100 x 100 22 against 37, 400 x 400 26 against 42, 640 x 640 (three
+    // quarters at rest) 43 against 45.
+    const size_t small = mixed(ctx) ? 640 * 640 : 256 * 256;
+    ctx->form = g.gravity == 0.0 && nc > small ? SALEC_STEP_FUSED : SALEC_STEP_PHASES;
     ctx->parity = 0;
     ctx->rates_valid = false;
     ctx->finalized = true;

@@ -14,14 +14,25 @@ namespace salec {
 // reached their end time are skipped; each run keeps its own dt reduction).
 // ---------------------------------------------------------------------------------
 
-// The FP64 phase 0 (equation of state per material, artificial viscosity) holds more live
-// values than 64 registers: with one resident block of the largest shape as its bound it
-// takes 80-90 registers and spills nothing (under the default bound ptxas settled on 64
-// and spilled 8-144 bytes a thread); the mixed form keeps the default.
-template <typename T> struct Phase0Bound { static constexpr int min_blocks = sizeof(T) == 8 ? 1 : 0; };
+// Registers a thread of a phase kernel may take.  The FP64 kernels are bound by the FP64 pipe
+// and keep what they need (80-94 for phase 0, no spills).  The mixed kernels are bound by
+// latency, so warps in flight count for more than the few bytes of spill a cap costs: on a
+// batch of 16 runs with two materials and strength (5.5e6 cells) phase 0 took 147 us at its
+// own 48 registers (56 % of the warps), 131 at 40 and 111 at 32 (91 %), phase 2 161 / 132 /
+// 120, the cell remap 251 at 56, 229 at 48, 223 at 40 and no less at 32; with three materials
+// the remap spills more and is best at 48 (the layered grid: 24.4 us at 56, 22.5 at 48, 26.1
+// at 40), with one hydrodynamic material at 32.
+enum Phase { kPh0, kPh1, kPh2, kPh3a, kPh3b };
+template <typename T, int NM, bool STR>
+constexpr int phase_regs(Phase ph)
+{
+    if (sizeof(T) == 8) return 128;
+    if (ph != kPh3a) return 32;
+    return NM == 3 ? 48 : NM == 2 || STR ? 40 : 32;
+}
 
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads, Phase0Bound<T>::min_blocks) k_phase0(ParamsT<T> P) { body_phase0<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh0))) k_phase0(ParamsT<T> P) { body_phase0<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T>
 __global__ void k_courant(ParamsT<T> P)
 {
@@ -37,20 +48,20 @@ cudaError_t launch_courant(const ParamsT<T>& P, cudaStream_t s)
 template cudaError_t launch_courant<double>(const ParamsT<double>&, cudaStream_t);
 template cudaError_t launch_courant<float>(const ParamsT<float>&, cudaStream_t);
 template <typename T, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) k_phase1(ParamsT<T> P) { body_phase1<T, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, 1, STR>(kPh1))) k_phase1(ParamsT<T> P) { body_phase1<T, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) k_phase2(ParamsT<T> P) { body_phase2<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh2))) k_phase2(ParamsT<T> P) { body_phase2<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) k_phase3a(ParamsT<T> P) { body_phase3a<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh3a))) k_phase3a(ParamsT<T> P) { body_phase3a<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads) k_phase3b(ParamsT<T> P) { body_phase3b<T>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, 1, false>(kPh3b))) k_phase3b(ParamsT<T> P) { body_phase3b<T>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T, int NM>
 __global__ void __launch_bounds__(kMaxThreads) k_phase3c(ParamsT<T> P) { body_phase3c<T, NM>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 
 // phase 0 decides for the whole step: a run at or past its end time, or one whose status
 // reports a failure (non-positive volume or density, NaN, dt below dt_min), does nothing
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads, Phase0Bound<T>::min_blocks) kb_phase0(const ParamsT<T>* __restrict__ runs,
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh0))) kb_phase0(const ParamsT<T>* __restrict__ runs,
                                                                                      const BatchTile* __restrict__ work)
 {
     const BatchTile w = work[blockIdx.x];
@@ -83,51 +94,20 @@ __global__ void kb_courant(const ParamsT<T>* __restrict__ runs, int nruns)
         CALL(P, w.bx, w.by, w.g & 0xffff, w.g >> 16);                                      \
     }
 template <typename T, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) kb_phase1(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, 1, STR>(kPh1))) kb_phase1(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase1, (body_phase1<T, STR, UNI>))
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) kb_phase2(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh2))) kb_phase2(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase2, (body_phase2<T, NM, STR, UNI>))
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) kb_phase3a(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh3a))) kb_phase3a(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase3a, (body_phase3a<T, NM, STR, UNI>))
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads) kb_phase3b(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
+__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, 1, false>(kPh3b))) kb_phase3b(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase3b, (body_phase3b<T>))
 template <typename T, int NM>
 __global__ void __launch_bounds__(kMaxThreads) kb_phase3c(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase3c, (body_phase3c<T, NM>))
-
-// The mixed form's remap kernels for one hydrodynamic material (and its vertex remap for
-// any material count, single and batched) are latency-bound (19-34 % of DRAM peak at
-// 62-75 % occupancy): their registers are capped so that a full SM of threads (4 blocks
-// of the largest shape) fits, at the cost of a few bytes of spill.  With more materials
-// or strength the cell remap would spill heavily under such a cap; the FP64 kernels are
-// bound by the FP64 pipe.  Both keep the compiler's own register choice.
-template <>
-__global__ void __launch_bounds__(kMaxThreads, 4) k_phase3a<float, 1, false, true>(ParamsT<float> P)
-{
-    body_phase3a<float, 1, false, true>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
-}
-template <>
-__global__ void __launch_bounds__(kMaxThreads, 4) k_phase3a<float, 1, false, false>(ParamsT<float> P)
-{
-    body_phase3a<float, 1, false, false>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
-}
-template <>
-__global__ void __launch_bounds__(kMaxThreads, 4) k_phase3b<float>(ParamsT<float> P)
-{
-    body_phase3b<float>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y);
-}
-template <>
-__global__ void __launch_bounds__(kMaxThreads, 4) kb_phase3b<float>(const ParamsT<float>* __restrict__ runs,
-                                                                   const BatchTile* __restrict__ work)
-{
-    const BatchTile w = work[blockIdx.x];
-    const ParamsT<float>& P = runs[w.run];
-    if (P.p.scal->active == 0) return;
-    body_phase3b<float>(P, w.bx, w.by, w.g & 0xffff, w.g >> 16);
-}
 
 // ---------------------------------------------------------------------------------
 // Read-out kernels

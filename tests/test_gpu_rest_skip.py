@@ -30,6 +30,7 @@ def test_tiles_copied_once_match_tiles_always_computed(nr, nz, kind, precision):
         spec["grid"]["dr"] = W.stretched_sizes(nr - 9, 10.0, 0, 9)
     names = FIELDS + (("srr", "szz", "srz", "D") if kind == "strength" else ())
     a, b = salec.Sim(spec, precision=precision), salec.Sim(spec, precision=precision)
+    a.step_form = b.step_form = "fused"
     b.set_rest_copy(0)
     for s in (a, b):
         s.step(5)
@@ -44,6 +45,7 @@ def test_tiles_copied_once_match_tiles_always_computed(nr, nz, kind, precision):
     image = a.get_state()
     a.step(20)
     c = salec.Sim(spec, precision=precision)
+    c.step_form = "fused"
     c.set_state(image)
     c.step(20)
     b.step(20)
