@@ -70,16 +70,23 @@ __device__ __forceinline__ unsigned long long global_ns()
     return t;
 }
 
-// bounded wait; false when the time limit ran out.  The clock is read only once the first
-// polls have failed: most waits of a pipeline end within them.
+// bounded wait; false when the time limit ran out
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
 {
-    for (int k = 0; k < 64; ++k)
-        if (mbar_try_wait(bar, parity)) return true;
     const unsigned long long t0 = global_ns();
     while (!mbar_try_wait(bar, parity))
         if (global_ns() - t0 > kWaitNs) return false;
     return true;
+}
+
+// the same for short waits on a critical path: the clock is only read once the first polls
+// have failed (where other warps of the SM compute meanwhile, reading it between polls is the
+// better use of the issue slots: the persistent forward kernel keeps mbar_wait)
+__device__ __forceinline__ bool mbar_wait_short(uint64_t* bar, uint32_t parity)
+{
+    for (int k = 0; k < 64; ++k)
+        if (mbar_try_wait(bar, parity)) return true;
+    return mbar_wait(bar, parity);
 }
 
 // True in one thread of the (converged) warp.  The tensor-core and bulk-copy instructions

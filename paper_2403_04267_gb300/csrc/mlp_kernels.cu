@@ -289,7 +289,7 @@ constexpr uint32_t kWStageBytes = kFusedHid * kBK * 2;     // 32768
 // The inference pass, persistent and warp-specialised: one CTA per SM takes 128-sample
 // tiles two at a time and alternates them, so that the tensor cores work on one tile while
 // the epilogue warps work on the other.  Per tile x (0, 1): an activation buffer H_x (BF16,
-// four 128-byte swizzled K slices, 64 KB) and a 256-column accumulator in tensor memory (both tiles: all
+// canonical K-major, 64 KB) and a 256-column accumulator in tensor memory (both tiles: all
 // 512 columns).  Warp 0 streams the weight slices (64-wide K slices, 256 rows x 128 bytes)
 // with TMA into a 2-stage ring, 128-byte swizzled; warp 1 issues the MMAs of job (x, layer)
 // once H_x holds that layer's input and frees each ring stage by tcgen05.commit; warps
@@ -333,7 +333,7 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
     __shared__ uint32_t tmem_holder;
     __shared__ volatile int abort_flag;
 
-    const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int G = gridDim.x;
     if (tid == 0) {
         for (int k = 0; k < kPPStages; ++k) { mbar_init(&wfull[k], 1); mbar_init(&wempty[k], 1); }
@@ -369,7 +369,7 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
 
     if (warp == 0) {
         // ---- weight producer ----
-        if (elect_one()) {
+        if (lane == 0) {
             int fills[kPPStages] = {0, 0};
             int stage = 0;
             for (int k = 0; k < npairs_mine && !abort_flag; ++k)
@@ -395,7 +395,7 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
         }
     } else if (warp == 1) {
         // ---- MMA issuer ----
-        if (elect_one()) {
+        if (lane == 0) {
             int used[kPPStages] = {0, 0}, hwait[2] = {0, 0}, commits[2] = {0, 0};
             int stage = 0;
             const uint32_t w1 = smem_u32(W1s);
@@ -410,18 +410,17 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
                         const uint32_t acc = tmem + (uint32_t)(x * kFusedHid);
                         const uint32_t hb = smem_u32(Hbuf + x * kHBytes);
                         if (l == 0) {
-                            mma_bf16(acc, sdesc_sw128(hb), sdesc(w1, kFusedHid * 16, 128), idesc, 0u);
+                            mma_bf16(acc, sdesc(hb, kBM * 16, 128), sdesc(w1, kFusedHid * 16, 128), idesc, 0u);
                         } else {
-                            // descriptors by addition: a K step is 32 bytes of a swizzled row
-                            uint64_t ad = sdesc_sw128(hb);
                             for (int kt = 0; kt < kFusedHid / kBK; ++kt) {
                                 if (!mbar_wait(&wfull[stage], (uint32_t)(used[stage]++) & 1u)) { abort_flag = 1; break; }
                                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                                const uint64_t bd = sdesc_sw128(smem_u32(Wring + stage * kWStageBytes));
+                                const uint32_t wb = smem_u32(Wring + stage * kWStageBytes);
 #pragma unroll
-                                for (int kk = 0; kk < kBK / 16; ++kk)
-                                    mma_bf16(acc, ad + kk * 2, bd + kk * 2, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
-                                ad += kSliceBytes >> 4;
+                                for (int kk = 0; kk < kBK / 16; ++kk) {
+                                    const uint64_t ad = sdesc(hb + (kt * (kBK / 8) + 2 * kk) * (kBM * 16), kBM * 16, 128);
+                                    mma_bf16(acc, ad, sdesc_sw128(wb + kk * 32), idesc, (kt > 0 || kk > 0) ? 1u : 0u);
+                                }
                                 mma_commit(&wempty[stage]);
                                 stage ^= 1;
                             }
@@ -443,15 +442,15 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
         int accw[2] = {0, 0};
         // the warp decides together: an abort seen by any lane ends the warp's loop
         auto aborted = [&]() { return __any_sync(0xffffffffu, abort_flag != 0); };
-        // inputs of tile t into H_x: X rows (8 BF16), K padded to 16
+        // inputs of tile t into H_x: X rows (8 BF16 = one core-matrix row), K padded to 16
         auto stage_inputs = [&](int x, int t) {
             if (cq == 0) {
                 const int m = t * kBM + r;
                 uint4 xv = make_uint4(0u, 0u, 0u, 0u);
                 if (m < a.B) xv = *reinterpret_cast<const uint4*>(a.X + (long)m * a.ld_x);
                 unsigned char* H = Hbuf + x * kHBytes;
-                *reinterpret_cast<uint4*>(H + sw128_off(r, 0)) = xv;
-                *reinterpret_cast<uint4*>(H + sw128_off(r, 1)) = make_uint4(0u, 0u, 0u, 0u);
+                *reinterpret_cast<uint4*>(H + cm_off(r, 0, kBM)) = xv;
+                *reinterpret_cast<uint4*>(H + cm_off(r, 1, kBM)) = make_uint4(0u, 0u, 0u, 0u);
             }
         };
         auto release = [&](int x) {
@@ -503,10 +502,8 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
                                     w[2 * qq + 1] = *reinterpret_cast<const uint32_t*>(&hi);
                                 }
                             }
-                            unsigned char* Hs = H + cq * kSliceBytes;       // columns 64 cq ..
-                            const int ch = (c0 & 63) >> 3;
-                            *reinterpret_cast<uint4*>(Hs + sw128_off(r, ch)) = make_uint4(w[0], w[1], w[2], w[3]);
-                            *reinterpret_cast<uint4*>(Hs + sw128_off(r, ch + 1)) = make_uint4(w[4], w[5], w[6], w[7]);
+                            *reinterpret_cast<uint4*>(H + cm_off(r, (c0 >> 3), kBM)) = make_uint4(w[0], w[1], w[2], w[3]);
+                            *reinterpret_cast<uint4*>(H + cm_off(r, (c0 >> 3) + 1, kBM)) = make_uint4(w[4], w[5], w[6], w[7]);
                         }
                         release(x);
                     } else {
