@@ -185,13 +185,13 @@ salec_status salec_step(salec_ctx* ctx, int nsteps);
  *                      stays at rest, or by a copy kernel beside it, every step:
  *                      salec_set_rest_copy), and the other tiles are queued for the tile
  *                      kernel (one CTA per resident slot of the device).
- *                      Default when grid->gravity == 0 on grids of more than 256 x 256 cells
- *                      (mixed form: 640 x 640), where many tiles keep the SMs busy.
+ *                      Default when grid->gravity == 0, in FP64 on grids of more than
+ *                      256 x 256 cells, where many tiles keep the SMs busy.
  *   SALEC_STEP_PHASES  six kernels over the whole grid and the Courant kernel, in place
  *                      (block shapes from salec_set_block_shapes / salec_autotune).
  *                      Default under gravity, where no tile is quiescent and this form,
- *                      which computes no cell twice, issues fewer instructions, and on
- *                      smaller grids.
+ *                      which computes no cell twice, issues fewer instructions, and in
+ *                      FP64 on smaller grids.
  * Both forms compute the same cycle with the same arithmetic per cell and vertex;
  * salec_set_step_form returns SALEC_EINVAL for another value, SALEC_EORDER before
  * salec_finalize. */

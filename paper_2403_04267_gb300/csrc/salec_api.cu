@@ -791,13 +791,13 @@ salec_status salec_finalize(salec_ctx* ctx)
     // nothing (4000 x 4000: mixed form 0.08 against 0.90 ms per step, FP64 0.29 against
     // 7.1).  Under gravity no tile is quiescent (a loaded column is not at zero pressure) and
     // the phase kernels, which compute no cell twice, are faster (the paper's layered grid:
-    // 0.054 against 0.087 ms, FP64 0.45 against 0.70).  So they are on small grids, whose few
-    // tiles leave most SMs idle while one SM works through a tile's frame: FP64 100 x 100
-    // 58 against 103 us per step, 250 x 250 72 against 94, 400 x 400 (half at rest) 119
-    // against 90; mixed 100 x 100 22 against 37, 400 x 400 26 against 42, 640 x 640 (three
-    // quarters at rest) 43 against 45.
-    const size_t small = mixed(ctx) ? 640 * 640 : 256 * 256;
-    ctx->form = g.gravity == 0.0 && nc > small ? SALEC_STEP_FUSED : SALEC_STEP_PHASES;
+    // 0.054 against 0.087 ms, FP64 0.45 against 0.70).  So they are in FP64 on small grids,
+    // whose few tiles leave most SMs idle while one SM works through a tile's frame: 100 x 100
+    // 37 against 103 us per step, 250 x 250 72 against 94, 400 x 400 (half at rest) 119
+    // against 90.  (The mixed form would gain too, 100 x 100 22 against 37, but its two forms
+    // round differently, and a run's FP32 results should not change with this choice.)
+    const bool small = !mixed(ctx) && nc <= 256 * 256;
+    ctx->form = g.gravity == 0.0 && !small ? SALEC_STEP_FUSED : SALEC_STEP_PHASES;
     ctx->parity = 0;
     ctx->rates_valid = false;
     ctx->finalized = true;

@@ -1,6 +1,6 @@
-"""The default step form by grid size (no gravity): the phase kernels up to 256 x 256 cells in
-FP64 and 640 x 640 in the mixed form, the fused form beyond; and in FP64 both forms agree
-with each other at the repository's parity bar (1e-9 of a field's maximum) on grids of a few
+"""The default step form by grid size (no gravity): in FP64 the phase kernels up to 256 x 256
+cells and the fused form beyond, in the mixed form always the fused form; and in FP64 both
+forms agree with each other at the repository's parity bar (1e-9 of a field's maximum) on grids of a few
 cells, at the rule's edge and with fractions of several materials in a cell."""
 import numpy as np
 import pytest
@@ -10,10 +10,10 @@ from paper_2403_04267_gb300 import salec, workloads as W
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("precision,side", [("fp64", 256), ("fp32mix", 640)])
-def test_default_form_by_size(precision, side):
-    for nr, form in ((side, "phases"), (side + 1, "fused")):
-        s = salec.Sim(W.impact(nr, side, 10.0, W.basalt(), None, 5, 9e3, int(0.7 * side), 16), precision=precision)
+@pytest.mark.parametrize("precision,small", [("fp64", "phases"), ("fp32mix", "fused")])
+def test_default_form_by_size(precision, small):
+    for nr, form in ((100, small), (256, small), (257, "fused")):
+        s = salec.Sim(W.impact(nr, 256, 10.0, W.basalt(), None, 5, 9e3, 179, 16), precision=precision)
         assert s.step_form == form and s.launches_per_step() == (7 if form == "phases" else 3)
     s = salec.Sim(W.impact(40, 40, 10.0, W.basalt(), None, 3, 9e3, 28, 4, gravity=1.62), precision=precision)
     assert s.step_form == "phases"
