@@ -77,15 +77,16 @@ def kernel_bytes_per_cell(e: int) -> dict:
         "k_phase3c": 2 * e + e + 8 + 8,                           # (f,rho) kheat I(rw)
         # the fused cycle reads and writes the persistent state once (plus the Courant kernel)
         "k_step_fused": step_bytes_per_cell(e),
-        # a tile at rest: (f, rho), I and the EoS cache (p, c^2) read and written, vertices
-        # written (at rest): the same count as the state's
+        # a tile that comes to rest is copied once: (f, rho), I and the EoS cache (p, c^2) read
+        # and written, vertices written (at rest): the same count as the state's
         "k_rest_tiles": 2 * (2 * e + 8 + 2 * e) + 2 * e,
-        # the same tiles moved by the copy kernel that runs beside the tile kernel
+        # the tiles at rest moved at every step by the copy kernel that runs beside the tile
+        # kernel
         "k_rest_copy": 2 * (2 * e + 8 + 2 * e) + 2 * e,
     }
 
 
-# the fused form's kernels that copy the tiles at rest (before the tile kernel, or beside it)
+# the fused form's kernels for the tiles at rest (before the tile kernel, or beside it)
 REST_KERNELS = ("k_rest_tiles", "k_rest_copy")
 
 
@@ -113,7 +114,9 @@ def _sm_max_mhz():
 
 
 class ClockSampler:
-    """nvidia-smi clocks and throttle reasons sampled every 200 ms while running."""
+    """nvidia-smi clocks and throttle reasons sampled every 20 ms while running.  Entering waits
+    for the first sample (at most 3 s), so that a timed region of a few milliseconds, right
+    after the warm-up, has one."""
 
     FIELDS = ("index,clocks.sm,clocks.max.sm,power.draw,clocks_event_reasons.active,"
               "clocks_event_reasons.hw_slowdown,clocks_event_reasons.hw_thermal_slowdown,"
@@ -130,7 +133,10 @@ class ClockSampler:
             os.close(fd)
             self.proc = subprocess.Popen(
                 ["nvidia-smi", "-i", str(self.gpu), f"--query-gpu={self.FIELDS}", "--format=csv,noheader,nounits",
-                 "-lms", "200"], stdout=open(self.path, "w"), stderr=subprocess.DEVNULL)
+                 "-lms", "20"], stdout=open(self.path, "w"), stderr=subprocess.DEVNULL)
+            t0 = time.perf_counter()
+            while os.path.getsize(self.path) == 0 and self.proc.poll() is None and time.perf_counter() - t0 < 3.0:
+                time.sleep(0.002)
         except Exception:
             self.proc = None
         return self
@@ -689,7 +695,8 @@ def _active(args, hbm_peak):
             q, t = sim.fused_queue()
             r["tiles_queued_last_step"] = [q, t]
         if prec == "fp32mix":
-            gbs = step_bytes_per_cell(4) * cells / (ms * 1e-3) / 1e9
+            frac = r["tiles_queued_last_step"][0] / r["tiles_queued_last_step"][1] if "tiles_queued_last_step" in r else 1.0
+            gbs = step_bytes_per_cell(4) * cells * frac / (ms * 1e-3) / 1e9
             r["step_hbm"] = {"achieved_gbs": round(gbs, 1), "peak_gbs": hbm_peak, "frac": round(gbs / hbm_peak, 4),
                              "bytes_per_cell": step_bytes_per_cell(4)}
         out[prec] = r
@@ -828,7 +835,7 @@ def main():
         queue = None
         if sim.step_form == "fused":
             # the same K steps again, untimed, one call each: how many tiles each step ran
-            # through the whole cycle (the others the rest-tile kernel copied)
+            # through the whole cycle (the others were at rest)
             sim.set_state(snap)
             qs = []
             for _ in range(args.steps):
@@ -881,18 +888,23 @@ def main():
         dom = dom or max(kt, key=kt.get)
         kb = kernel_bytes_per_cell(e)
         # cells one launch processes: every cell for a phase kernel; in the fused form the
-        # cells of the tiles at rest (rest-tile kernel) or of the queued tiles (tile kernel),
-        # averaged over the K steps
+        # cells of the queued tiles (tile kernel) or of the tiles at rest (copy kernel beside
+        # it), averaged over the K steps; the rest-tile kernel only tests tiles that stay at
+        # rest, so no bytes are counted for it
         units = float(cells)
         q = res.get("queue")
         if q:
             qf = q["queued_mean"] / q["tiles"]
-            units = cells * (1.0 - qf if dom in REST_KERNELS else qf)
+            units = 0.0 if dom == "k_rest_tiles" else cells * (1.0 - qf if dom in REST_KERNELS else qf)
         gbs = kb[dom] * units / (kt[dom] * 1e-3) / 1e9
         roof = {"kernel": dom, "hbm": {"achieved_gbs": round(gbs, 1), "peak_gbs": hbm_peak, "peak_kind": peak_kind,
                                        "frac": round(gbs / hbm_peak, 4), "bytes_per_cell": kb[dom],
                                        "cells_per_launch": round(units)}}
         return roof, dom
+
+    def moved_cells(res):
+        q = res.get("queue")
+        return cells * q["queued_mean"] / q["tiles"] if q else cells
 
     res64 = measure("fp64", not args.no_e2e) if args.precision in ("both", "fp64") else None
     # the FP64 form's other step form beside the library's choice
@@ -957,7 +969,7 @@ def main():
         else:
             roof = alu_roof(dom)
             roof["hbm"] = roof_hbm["hbm"]
-        if rest_k is not None and dom != rest_k:
+        if rest_k == "k_rest_copy" and dom != rest_k:
             rr, _ = roofline(main_res, e_main, rest_k)
             line_rest = hbm_roof(rr, rest_k, "fp64")
         else:
@@ -978,7 +990,9 @@ def main():
                    "sim_time_s": sc["t"], "status": sc["status"]},
         "gpu_launches": main_res["launches"],
         "kernel_ms": {k: round(v, 4) for k, v in main_res["ktimes"].items()},
-        "step_hbm_frac": round(step_bytes_per_cell(e_main) * cells / (ms / args.steps * 1e-3) / 1e9 / hbm_peak, 4),
+        # the state of the cells a step works on (fused form: the queued tiles'; a tile at rest
+        # is not moved), read and written once
+        "step_hbm_frac": round(step_bytes_per_cell(e_main) * moved_cells(main_res) / (ms / args.steps * 1e-3) / 1e9 / hbm_peak, 4),
         "roofline": roof, "clocks": main_res["clocks"], "e2e": main_res.get("e2e"), "step_form": main_res["form"],
     }
     if fp64_alu is not None:
@@ -1005,7 +1019,7 @@ def main():
             "speedup_vs_fp64": res32["value"] / res64["value"], "step_form": res32["form"],
             "kernel_ms": {k: round(v, 4) for k, v in res32["ktimes"].items()},
             "roofline": hbm_roof(r32, d32, "fp32mix"), "fused_queue": res32.get("queue"),
-            "step_hbm_frac": round(step_bytes_per_cell(4) * cells / (res32["ms"] / args.steps * 1e-3) / 1e9 / hbm_peak, 4),
+            "step_hbm_frac": round(step_bytes_per_cell(4) * moved_cells(res32) / (res32["ms"] / args.steps * 1e-3) / 1e9 / hbm_peak, 4),
             "peak_pressure_decay_vs_fp64_same_steps": dec,
             "gpu_launches": res32["launches"], "clocks": res32["clocks"], "status": res32["scalars"]["status"]}
         if res32f is not None:
@@ -1014,7 +1028,7 @@ def main():
                 "value": res32f["value"], "unit": UNIT, "ms_per_step": res32f["ms_max"] / args.steps,
                 "kernel_ms": {k: round(v, 4) for k, v in res32f["ktimes"].items()},
                 "roofline": hbm_roof(rf, df, "fp32mix"),
-                "step_hbm_frac": round(step_bytes_per_cell(4) * cells / (res32f["ms"] / args.steps * 1e-3) / 1e9 / hbm_peak, 4),
+                "step_hbm_frac": round(step_bytes_per_cell(4) * moved_cells(res32f) / (res32f["ms"] / args.steps * 1e-3) / 1e9 / hbm_peak, 4),
                 "gpu_launches": res32f["launches"], "status": res32f["scalars"]["status"]}
         if not args.no_accuracy and ws == 1:
             line["fp32_mix"]["accuracy"] = _fp32_accuracy(args)
@@ -1043,9 +1057,9 @@ _FLOPS_PER_CELL: dict = {"k_phase0": 85.1, "k_phase1": 37.7, "k_phase2": 27.4, "
 _TRAFFIC_PER_CELL: dict = {"k_phase0": 57.7, "k_phase1": 72.2, "k_phase2": 75.3, "k_phase3a": 78.5, "k_phase3b": 62.8, "k_phase3c": 22.1}
 _TRAFFIC_PER_CELL_FP32MIX: dict = {"k_phase0": 27.7, "k_phase1": 30.8, "k_phase2": 40.1, "k_phase3a": 42.3, "k_phase3b": 29.6, "k_phase3c": 10.8}
 # fraction of the FP64 pipe's issue slots each FP64-form kernel keeps busy (ncu,
-# sm__pipe_fp64_cycles_active, 2000 x 2000, the fused kernels at the second timed step)
+# sm__pipe_fp64_cycles_active, 2000 x 2000; the fused kernels 4000 x 4000, the run's first step)
 _FP64_PIPE_BUSY: dict = {"k_phase0": 0.847, "k_phase1": 0.847, "k_phase2": 0.845, "k_phase3a": 0.847, "k_phase3b": 0.841,
-                         "k_phase3c": 0.783, "k_step_fused": 0.735, "k_rest_tiles": 0.180}
+                         "k_phase3c": 0.783, "k_step_fused": 0.72, "k_rest_tiles": 0.12}
 # The fused form's two kernels on the headline workload (4000 x 4000, K = 20 timed steps after
 # W = 5 warm-up steps): DRAM read + write bytes and FP64 operations per launch, the mean over
 # the 20 launches of the timed region from one-pass ncu captures of the same command
@@ -1053,12 +1067,13 @@ _FP64_PIPE_BUSY: dict = {"k_phase0": 0.847, "k_phase1": 0.847, "k_phase2": 0.845
 # for that case only.
 _FULL_SIZE_CASE = ("large_4000", 20, 5)
 _FUSED_FULL_SIZE: dict = {
-    "fp64": {"k_rest_tiles": {"traffic": 1.43016e9}, "k_step_fused": {"traffic": 4.2122e7, "flops": 1.14608e8}},
-    "fp32mix": {"k_rest_tiles": {"traffic": 8.0653e8}, "k_step_fused": {"traffic": 2.6158e7}},
+    "fp64": {"k_rest_tiles": {"traffic": 3.0415e5}, "k_step_fused": {"traffic": 4.2143e7, "flops": 1.02645e8}},
+    "fp32mix": {"k_rest_tiles": {"traffic": 1.5863e5}, "k_step_fused": {"traffic": 2.6142e7}},
 }
 # kernels changed since their counters were taken: neither DRAM traffic nor flop rates are
 # reported for them until the next capture
-_COUNTERS_STALE: dict = {"fp64": set(), "fp32mix": set()}
+_COUNTERS_STALE: dict = {"fp64": {"k_phase0", "k_phase1", "k_phase2", "k_phase3a"},
+                         "fp32mix": {"k_phase0", "k_phase2", "k_phase3a"}}
 # Beside the copy kernel (salec_set_rest_copy mode 2) the FP64 tile kernel is another
 # instantiation (120 registers, the same arithmetic) sharing the SMs with the copies: its
 # FP64 operation count carries over, the DRAM traffic of the capture above does not.
