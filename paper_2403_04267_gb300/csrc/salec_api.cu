@@ -1425,6 +1425,7 @@ struct salec_batch {
     bool pgraph = true;             // its launch is captured in the chunk graph (false: capture refused)
     size_t off_sync = 0;            // its grid barrier
     bool expire_next = false;       // salec_batch_expire_next_barrier
+    cudaEvent_t home = nullptr;     // a run's copies into its first copy, for the batch's stream to wait for
 };
 
 static salec_status bfail(salec_batch* b, salec_status st, const char* msg)
@@ -1485,6 +1486,8 @@ salec_status salec_batch_bytes(salec_ctx* const* runs, int nruns, size_t* bytes)
     return SALEC_OK;
 }
 
+static salec_status batch_fields(salec_batch* b);
+
 static salec_status batch_build_work(salec_batch* b)
 {
     b->retired.resize(b->runs.size(), 0);
@@ -1514,8 +1517,6 @@ salec_status salec_batch_create(salec_ctx* const* runs, int nruns, void* dev_buf
 {
     salec_status st = batch_check(runs, nruns);
     if (st != SALEC_OK || !out) return st != SALEC_OK ? st : SALEC_EINVAL;
-    for (int r = 0; r < nruns; ++r)
-        if ((st = current_fields(runs[r], true)) != SALEC_OK) return st;
     salec_batch* b = new salec_batch();
     const size_t need = batch_layout(runs, nruns, b);
     if (!dev_buf || bytes < need || ((uintptr_t)dev_buf % kAlign) != 0) { delete b; return SALEC_ENOMEM; }
@@ -1529,6 +1530,8 @@ salec_status salec_batch_create(salec_ctx* const* runs, int nruns, void* dev_buf
     b->dev = (char*)dev_buf;
     b->bytes = bytes;
     for (int k = 0; k < 6; ++k) b->shape[k] = kDefaultShape;
+    st = batch_fields(b);
+    if (st != SALEC_OK) { salec_batch_destroy(b); return st; }
     // run parameter blocks
     cudaError_t e = cudaSuccess;
     if (b->precision == SALEC_FP32MIX) {
@@ -1542,9 +1545,9 @@ salec_status salec_batch_create(salec_ctx* const* runs, int nruns, void* dev_buf
         e = cudaMemcpyAsync(b->dev + b->off_params, P.data(), P.size() * sizeof(P[0]), cudaMemcpyHostToDevice, b->stream);
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     }
-    if (e != cudaSuccess) { delete b; return SALEC_ECUDA; }
+    if (e != cudaSuccess) { salec_batch_destroy(b); return SALEC_ECUDA; }
     st = batch_build_work(b);
-    if (st != SALEC_OK) { delete b; return st; }
+    if (st != SALEC_OK) { salec_batch_destroy(b); return st; }
     *out = b;
     return SALEC_OK;
 }
@@ -1593,11 +1596,19 @@ static salec_status batch_prepare_persistent(salec_batch* b)
 static salec_status batch_restore_retired(salec_batch* b);
 
 // a run stepped alone in the fused form since the last batched step has its fields in the
-// second copy: bring them back (the batch's kernels work in place on the first)
+// second copy: bring them back (the batch's kernels work in place on the first).  The copies
+// go on the run's stream, behind its steps; the batch's stream waits for them.
 static salec_status batch_fields(salec_batch* b)
 {
-    for (salec_ctx* r : b->runs)
+    for (salec_ctx* r : b->runs) {
+        const bool moves = r->parity != 0;
         if (salec_status st = current_fields(r, true)) return bfail(b, st, r->err.c_str());
+        if (!moves || r->stream == b->stream) continue;
+        cudaError_t e = b->home ? cudaSuccess : cudaEventCreateWithFlags(&b->home, cudaEventDisableTiming);
+        if (e == cudaSuccess) e = cudaEventRecord(b->home, r->stream);
+        if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->home, 0);
+        if (e != cudaSuccess) return bfail(b, SALEC_ECUDA, cudaGetErrorString(e));
+    }
     return SALEC_OK;
 }
 
@@ -1885,6 +1896,7 @@ void salec_batch_destroy(salec_batch* b)
     if (!b) return;
     if (b->graph) cudaGraphExecDestroy(b->graph);
     for (cudaEvent_t e : b->ev) cudaEventDestroy(e);
+    if (b->home) cudaEventDestroy(b->home);
     delete b;
 }
 
