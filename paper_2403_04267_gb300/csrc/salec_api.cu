@@ -191,6 +191,7 @@ struct salec_ctx {
     int form = SALEC_STEP_PHASES;
     int parity = 0;                       // 1: the current fields are in the second copy
     bool rates_valid = false;             // the running Courant maximum holds the current state's rates
+    bool max_left = false;                // it may hold rates that the next phase 0 must not start from
     ParamsT<double> Pd_alt;               // the FP64 / mixed parameters reading the second copy
     ParamsT<float> Pf_alt;
     OutPtrsT<double> Od[2];               // where a fused step from copy k writes (the other copy)
@@ -339,6 +340,22 @@ static cudaError_t canonical(salec_ctx* ctx)
                             cudaMemcpyDeviceToDevice, ctx->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(ctx->base + L.work, 0, sizeof(TileWork), ctx->stream);
     if (e == cudaSuccess) ctx->parity = 0;
+    return e;
+}
+
+static cudaError_t clear_maximum(salec_ctx* ctx)
+{
+    return cudaMemsetAsync(ctx->base + ctx->L.scal + offsetof(DevScalars, maxbits), 0, sizeof(unsigned long long), ctx->stream);
+}
+
+// Phase 0 adds to a running maximum that its own Courant kernel leaves at zero.  A fused step
+// leaves the rates of its last state there, a checkpoint of a fused run brings them along, and
+// a host write can change the state under them: cleared before phases or batched steps follow.
+static cudaError_t drop_maximum(salec_ctx* ctx)
+{
+    if (!ctx->max_left) return cudaSuccess;
+    const cudaError_t e = clear_maximum(ctx);
+    if (e == cudaSuccess) ctx->max_left = false;
     return e;
 }
 
@@ -880,8 +897,7 @@ static salec_status step_fused(salec_ctx* ctx, int nsteps)
     if (!ctx->rates_valid) {
         const Layout& L = ctx->L;
         cudaError_t e = canonical(ctx);
-        if (e == cudaSuccess)
-            e = cudaMemsetAsync(ctx->base + L.scal + offsetof(DevScalars, maxbits), 0, sizeof(unsigned long long), ctx->stream);
+        if (e == cudaSuccess) e = clear_maximum(ctx);
         if (e == cudaSuccess) e = cudaMemsetAsync(ctx->base + L.rest[0], 0, L.work + 2 * sizeof(TileWork) - L.rest[0], ctx->stream);
         if (e == cudaSuccess && ctx->rest_copy) e = cudaMemsetAsync(ctx->base + L.rest[0], 1, L.ntiles, ctx->stream);
         unsigned char* rest0 = ctx->rest_copy ? at<unsigned char>(ctx, L.rest[0]) : nullptr;
@@ -889,6 +905,7 @@ static salec_status step_fused(salec_ctx* ctx, int nsteps)
                                              : launch_courant_rates<double>(ctx->Pd, rest0, ctx->stream);
         if (e != cudaSuccess) return cuda_check(ctx, e, "Courant rates");
         ctx->rates_valid = true;
+        ctx->max_left = true;
     }
     if (!ctx->timing && nsteps >= kGraphChunk && ctx->fgraph_ok) {
         const int p0 = ctx->parity;
@@ -932,7 +949,11 @@ salec_status salec_step(salec_ctx* ctx, int nsteps)
     if (ctx->form == SALEC_STEP_FUSED) return step_fused(ctx, nsteps);
     cudaError_t ce = canonical(ctx);
     if (ce != cudaSuccess) return cuda_check(ctx, ce, "canonical copy");
-    if (nsteps > 0) ctx->rates_valid = false;
+    if (nsteps > 0) {
+        ctx->rates_valid = false;
+        ce = drop_maximum(ctx);
+        if (ce != cudaSuccess) return cuda_check(ctx, ce, "Courant maximum");
+    }
     // whole chunks as graph replays (the kernel arguments are fixed after finalize; the
     // graph is captured again when the block shapes change)
     if (!ctx->timing && nsteps >= kGraphChunk && ctx->graph_ok) {
@@ -1141,7 +1162,10 @@ static salec_status current_fields(salec_ctx* ctx, bool write)
 {
     const cudaError_t e = canonical(ctx);
     if (e != cudaSuccess) return cuda_check(ctx, e, "canonical copy");
-    if (write) ctx->rates_valid = false;
+    if (write) {
+        ctx->rates_valid = false;
+        ctx->max_left = true;
+    }
     return SALEC_OK;
 }
 
@@ -1324,6 +1348,7 @@ salec_status salec_state_changed(salec_ctx* ctx)
     if (!ctx->finalized) return fail(ctx, SALEC_EORDER, "state_changed before finalize");
     ctx->parity = 0;
     ctx->rates_valid = false;
+    ctx->max_left = true;
     return SALEC_OK;
 }
 
@@ -1596,14 +1621,17 @@ static salec_status batch_prepare_persistent(salec_batch* b)
 static salec_status batch_restore_retired(salec_batch* b);
 
 // a run stepped alone in the fused form since the last batched step has its fields in the
-// second copy: bring them back (the batch's kernels work in place on the first).  The copies
-// go on the run's stream, behind its steps; the batch's stream waits for them.
+// second copy: bring them back (the batch's kernels work in place on the first).  The copies,
+// and the clearing of a Courant maximum left over, go on the run's stream, behind its steps;
+// the batch's stream waits for them.
 static salec_status batch_fields(salec_batch* b)
 {
     for (salec_ctx* r : b->runs) {
-        const bool moves = r->parity != 0;
-        if (salec_status st = current_fields(r, true)) return bfail(b, st, r->err.c_str());
-        if (!moves || r->stream == b->stream) continue;
+        const bool queued = r->parity != 0 || r->max_left;
+        if (salec_status st = current_fields(r, false)) return bfail(b, st, r->err.c_str());
+        r->rates_valid = false;
+        if (salec_status st = cuda_check(r, drop_maximum(r), "Courant maximum")) return bfail(b, st, r->err.c_str());
+        if (!queued || r->stream == b->stream) continue;
         cudaError_t e = b->home ? cudaSuccess : cudaEventCreateWithFlags(&b->home, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventRecord(b->home, r->stream);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(b->stream, b->home, 0);
