@@ -1690,23 +1690,6 @@ cudaError_t launch_step_fused(const ParamsT<T>& P, const OutPtrsT<T>& O, cudaStr
 
 // ---- host side of the copy beside the tile kernel -----------------------------------------
 
-TmaEncodeTiledFn tma_encode_tiled()
-{
-    static TmaEncodeTiledFn fn = nullptr;
-    static bool tried = false;
-    if (!tried) {
-        tried = true;
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<TmaEncodeTiledFn>(p);
-        else
-            (void)cudaGetLastError();
-    }
-    return fn;
-}
-
 namespace {
 
 // the one instantiation whose tile-kernel CTA leaves room for a copy CTA on its SM (120

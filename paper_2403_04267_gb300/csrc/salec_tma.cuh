@@ -98,6 +98,19 @@ __device__ __forceinline__ void bulk_wait_all() { asm volatile("cp.async.bulk.wa
 typedef CUresult (*TmaEncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                      const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                      CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-TmaEncodeTiledFn tma_encode_tiled();
+inline TmaEncodeTiledFn tma_encode_tiled()
+{
+    // looked up once; a thread that comes while another looks it up waits for the result
+    static const TmaEncodeTiledFn fn = [] {
+        void* p = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &p, 12000, cudaEnableDefault, &q) == cudaSuccess &&
+            q == cudaDriverEntryPointSuccess)
+            return reinterpret_cast<TmaEncodeTiledFn>(p);
+        (void)cudaGetLastError();
+        return TmaEncodeTiledFn(nullptr);
+    }();
+    return fn;
+}
 
 }  // namespace salec
