@@ -99,19 +99,39 @@ struct Geo {
 // work on the FP64 pipe.  An upper bound in FP32 (from the high words, integer
 // instructions) decides first: warps none of whose cells can exceed the maximum seen so far
 // skip the FP64 evaluation.  The maximum that results is the same.
-__device__ __forceinline__ float up_f32(double x)       // >= |x|; +inf for NaN and beyond FP32
+__host__ __device__ __forceinline__ int high_word(double x)
 {
-    const int h = __double2hiint(x) & 0x7fffffff;
-    if (h < 0x38200000) return 1.2e-38f;
-    if (h >= 0x47e00000) return __int_as_float(0x7f800000);
-    return __int_as_float(((h - 0x38000000) << 3) + 16);
+#ifdef __CUDA_ARCH__
+    return __double2hiint(x);
+#else
+    long long b;
+    memcpy(&b, &x, 8);
+    return (int)(b >> 32);
+#endif
 }
-__device__ __forceinline__ float down_f32(double x)     // <= x for x >= 0
+__host__ __device__ __forceinline__ float f32_of_bits(int b)
 {
-    const int h = __double2hiint(x);
+#ifdef __CUDA_ARCH__
+    return __int_as_float(b);
+#else
+    float f;
+    memcpy(&f, &b, 4);
+    return f;
+#endif
+}
+__host__ __device__ __forceinline__ float up_f32(double x)       // >= |x|; +inf for NaN and from 2^127 on
+{
+    const int h = high_word(x) & 0x7fffffff;
+    if (h < 0x38200000) return 2.4e-38f;                         // below 2^-125 = 2.351e-38
+    if (h >= 0x47e00000) return f32_of_bits(0x7f800000);
+    return f32_of_bits(((h - 0x38000000) << 3) + 16);
+}
+__host__ __device__ __forceinline__ float down_f32(double x)     // <= x for x >= 0
+{
+    const int h = high_word(x);
     if (h < 0x38200000) return 0.0f;
-    if (h >= 0x47e00000) return 3.0e38f;
-    return __int_as_float((h - 0x38000000) << 3);
+    if (h >= 0x47e00000) return 1.7e38f;                         // from 2^127 = 1.701e38 on
+    return f32_of_bits((h - 0x38000000) << 3);
 }
 __device__ __forceinline__ float up_w(double2 v)
 {
