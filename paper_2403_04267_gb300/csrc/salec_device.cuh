@@ -151,13 +151,14 @@ __device__ __forceinline__ bool rate_may_raise(T2 va, T2 vb, T2 vc, T2 vd, T c2,
     return !(r <= down_f32(run));
 }
 
-// a / b with y = 1 / b (within an ulp): the quotient corrected by its exact remainder
-// (Markstein, IBM J. Res. Dev. 34, 1990), three instructions on the FP64 pipe instead of a
-// division's ten; exactly 1 for a == b
-__device__ __forceinline__ double div_by(double a, double b, double y)
+// a / b with y close to 1 / b (a few units in the last place: on a non-uniform grid both y and b
+// are products, each rounded): the quotient corrected by its remainder (Markstein, IBM J. Res.
+// Dev. 34, 1990), three instructions on the FP64 pipe instead of a division's ten.  Exactly 1
+// for a == b, otherwise within 0.5 + 2^-40 units in the last place of the true quotient.
+__host__ __device__ __forceinline__ double div_by(double a, double b, double y)
 {
     const double q = a * y;
-    return __fma_rn(__fma_rn(-q, b, a), y, q);
+    return fma(fma(-q, b, a), y, q);
 }
 __device__ __forceinline__ float div_by(float a, float b, float) { return a / b; }
 

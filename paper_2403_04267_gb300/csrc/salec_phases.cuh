@@ -652,7 +652,7 @@ __device__ __forceinline__ void body_phase3a(const ParamsT<T>& P, int bx, int by
         for (int m = 0; m < NM; ++m) {
             fnew[m] = zero;
             if (ByMat<T, NM>::value && !(use >> m & 1u)) continue;
-            // the rounded quotient: exact 1 for a full resting cell
+            // exactly 1 for a full resting cell
             fnew[m] = div_by(Vm[m], Vc, Geo<T, UNI>::ivol(P, i, j));
             if (fnew[m] < P.f_min) {
                 if (warp_any(nonzero(Mm[m])) && nonzero(Mm[m])) t_disc += double(Mm[m]);
