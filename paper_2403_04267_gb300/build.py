@@ -45,7 +45,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     for src in SOURCES:
         obj = os.path.join(BUILD, src.replace(".cu", ".o"))
         cmd = [nvcc(), "-c", "-Xcompiler", "-fPIC", "-Xcompiler", "-ffp-contract=off", "-std=c++17",
-               *ARCH, "-O3", "-lineinfo", "-diag-suppress", "1444", "-o", obj, os.path.join(CSRC, src)]
+               *ARCH, "-O3", "-lineinfo", "-o", obj, os.path.join(CSRC, src)]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((subprocess.Popen(cmd), cmd))

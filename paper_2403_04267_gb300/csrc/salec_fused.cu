@@ -147,18 +147,8 @@ __device__ __forceinline__ void store_pair(T4* a, int half, T2 v) { reinterpret_
 
 }  // namespace
 
-// Registers a thread of the tile kernel may take: what its occupancy leaves (65536 per SM),
-// or REGS where that is set (the instantiation that runs beside the copy kernel keeps 120
-// of its 128, so that its 16 warps leave room on the SM for the copy warp).
-template <int NT, int MINB, int REGS>
-struct TileRegs {
-    static constexpr int all = 65536 / (NT * MINB);
-    static constexpr int value = REGS ? REGS : (all > 255 ? 255 : all);
-};
-
-template <typename T, int NM, bool STR, bool UNI, int TW, int TH, int NT, int MINB, int REGS = 0>
-__global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS>::value))
-    k_step_fused(const ParamsT<T> P, const OutPtrsT<T> O)
+template <typename T, int NM, bool STR, bool UNI, int TW, int TH, int NT>
+__device__ __forceinline__ void body_step_fused(const ParamsT<T>& P, const OutPtrsT<T>& O)
 {
     typedef VT<T> V;
     typedef typename V::T2 T2;
@@ -1064,6 +1054,22 @@ __global__ void __launch_bounds__(NT, MINB) __maxnreg__((TileRegs<NT, MINB, REGS
     }
 }
 
+template <typename T, int NM, bool STR, bool UNI, int TW, int TH, int NT, int MINB>
+__global__ void __launch_bounds__(NT, MINB) k_step_fused(const ParamsT<T> P, const OutPtrsT<T> O)
+{
+    body_step_fused<T, NM, STR, UNI, TW, TH, NT>(P, O);
+}
+
+// The tile kernel beside the copy kernel: of the 128 registers a thread that its 512 threads
+// leave it takes at most 120 (118), so that the copy warp finds room on the SM.  A kernel of
+// its own: the compiler does not take __maxnreg__ beside __launch_bounds__.
+constexpr int kBesideRegs = 120;
+template <typename T, int NM, bool STR, bool UNI, int TW, int TH, int NT>
+__global__ void __maxnreg__(kBesideRegs) k_step_fused_beside(const ParamsT<T> P, const OutPtrsT<T> O)
+{
+    body_step_fused<T, NM, STR, UNI, TW, TH, NT>(P, O);
+}
+
 // A tile is at rest when it and its eight neighbours (those inside the grid) took the
 // quiescent path in the step that wrote the copy read here.
 __device__ __forceinline__ bool tile_at_rest(const unsigned char* __restrict__ rest_in, int tile, int nbx, int nby)
@@ -1695,7 +1701,7 @@ namespace {
 // the one instantiation whose tile-kernel CTA leaves room for a copy CTA on its SM (120
 // registers a thread, 110 KB of shared memory): FP64, one hydrodynamic material, uniform grid
 typedef Fused<double, 1, false, true> Beside;
-constexpr int kBesideTW = Beside::S::TW, kBesideTH = Beside::S::TH, kBesideRegs = 120;
+constexpr int kBesideTW = Beside::S::TW, kBesideTH = Beside::S::TH;
 constexpr int kCopyStageBytes = 2 * kBesideTW * kBesideTH * 16 + kBesideTW * kBesideTH * 8;
 constexpr int kCopySmemNeed = kCopyStages * kCopyStageBytes + kBesideTW * kBesideTH * 16 + 128;
 
@@ -1718,7 +1724,7 @@ bool map_2d(CUtensorMap* map, const void* base, long width, long rows, long pitc
 bool prepare_rest_copy(const ParamsT<double>& P, const OutPtrsT<double>& O, RestCopy* rc)
 {
     if (!rc || P.nmat != 1 || P.any_strength || !P.uniform || (P.nr & 1)) return false;
-    auto tile_k = k_step_fused<double, 1, false, true, kBesideTW, kBesideTH, Beside::S::NT, Beside::S::MINB, kBesideRegs>;
+    auto tile_k = k_step_fused_beside<double, 1, false, true, kBesideTW, kBesideTH, Beside::S::NT>;
     auto copy_k = k_rest_copy<1, kBesideTW, kBesideTH>;
     auto scan_k = k_rest_scan<kBesideTW, kBesideTH>;
     cudaFuncAttributes ft, fc;
@@ -1802,7 +1808,7 @@ cudaError_t launch_step_fused_beside(const ParamsT<double>& P, const OutPtrsT<do
     }
     if (ev) cudaEventRecord(ev[2], s);
     if (e == cudaSuccess) {
-        k_step_fused<double, 1, false, true, kBesideTW, kBesideTH, Beside::S::NT, Beside::S::MINB, kBesideRegs>
+        k_step_fused_beside<double, 1, false, true, kBesideTW, kBesideTH, Beside::S::NT>
             <<<O.ctas, Beside::S::NT, Beside::L::bytes, s>>>(P, O);
         e = cudaGetLastError();
     }

@@ -14,25 +14,32 @@ namespace salec {
 // reached their end time are skipped; each run keeps its own dt reduction).
 // ---------------------------------------------------------------------------------
 
-// Registers a thread of a phase kernel may take.  The FP64 kernels are bound by the FP64 pipe
-// and keep what they need (80-94 for phase 0, no spills).  The mixed kernels are bound by
+// Registers a thread of a phase kernel may take, set by the blocks of kMaxThreads that have to
+// fit an SM (the minimum of __launch_bounds__).  The FP64 kernels are bound by the FP64 pipe:
+// phase 0 keeps what it needs (84-94, batched 94-104, no spills; left to itself the compiler
+// takes 64 and spills up to 200 bytes), the others do best as the compiler chooses (with room
+// for 128 they take 4 to 16 more, and an 800 x 800 step of two materials with strength 4 %
+// longer).  The mixed kernels are bound by
 // latency, so warps in flight count for more than the few bytes of spill a cap costs: on a
 // batch of 16 runs with two materials and strength (5.5e6 cells) phase 0 took 147 us at its
 // own 48 registers (56 % of the warps), 131 at 40 and 111 at 32 (91 %), phase 2 161 / 132 /
 // 120, the cell remap 251 at 56, 229 at 48, 223 at 40 and no less at 32; with three materials
 // the remap spills more and is best at 48 (the layered grid: 24.4 us at 56, 22.5 at 48, 26.1
-// at 40), with one hydrodynamic material at 32.
+// at 40), with one hydrodynamic material at 32.  Four blocks leave 32 registers, three 40; 48
+// lie between three and two, so the mixed remap of three materials has a cap of its own
+// (__maxnreg__, which the compiler does not take beside __launch_bounds__) in kernels of its
+// own.
 enum Phase { kPh0, kPh1, kPh2, kPh3a, kPh3b };
 template <typename T, int NM, bool STR>
-constexpr int phase_regs(Phase ph)
+constexpr int phase_blocks(Phase ph)
 {
-    if (sizeof(T) == 8) return 128;
-    if (ph != kPh3a) return 32;
-    return NM == 3 ? 48 : NM == 2 || STR ? 40 : 32;
+    if (sizeof(T) == 8) return ph == kPh0 ? 1 : 0;
+    return ph == kPh3a && (NM > 1 || STR) ? 3 : 4;
 }
+constexpr int kRemap3Regs = 48;
 
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh0))) k_phase0(ParamsT<T> P) { body_phase0<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, NM, STR>(kPh0))) k_phase0(ParamsT<T> P) { body_phase0<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T>
 __global__ void k_courant(ParamsT<T> P)
 {
@@ -48,20 +55,23 @@ cudaError_t launch_courant(const ParamsT<T>& P, cudaStream_t s)
 template cudaError_t launch_courant<double>(const ParamsT<double>&, cudaStream_t);
 template cudaError_t launch_courant<float>(const ParamsT<float>&, cudaStream_t);
 template <typename T, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, 1, STR>(kPh1))) k_phase1(ParamsT<T> P) { body_phase1<T, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, 1, STR>(kPh1))) k_phase1(ParamsT<T> P) { body_phase1<T, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh2))) k_phase2(ParamsT<T> P) { body_phase2<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, NM, STR>(kPh2))) k_phase2(ParamsT<T> P) { body_phase2<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh3a))) k_phase3a(ParamsT<T> P) { body_phase3a<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, NM, STR>(kPh3a))) k_phase3a(ParamsT<T> P) { body_phase3a<T, NM, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, 1, false>(kPh3b))) k_phase3b(ParamsT<T> P) { body_phase3b<T>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, 1, false>(kPh3b))) k_phase3b(ParamsT<T> P) { body_phase3b<T>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 template <typename T, int NM>
 __global__ void __launch_bounds__(kMaxThreads) k_phase3c(ParamsT<T> P) { body_phase3c<T, NM>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
+
+template <bool STR, bool UNI>
+__global__ void __maxnreg__(kRemap3Regs) k_phase3a_three(ParamsT<float> P) { body_phase3a<float, 3, STR, UNI>(P, blockIdx.x, blockIdx.y, gridDim.x, gridDim.y); }
 
 // phase 0 decides for the whole step: a run at or past its end time, or one whose status
 // reports a failure (non-positive volume or density, NaN, dt below dt_min), does nothing
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh0))) kb_phase0(const ParamsT<T>* __restrict__ runs,
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, NM, STR>(kPh0))) kb_phase0(const ParamsT<T>* __restrict__ runs,
                                                                                      const BatchTile* __restrict__ work)
 {
     const BatchTile w = work[blockIdx.x];
@@ -94,16 +104,22 @@ __global__ void kb_courant(const ParamsT<T>* __restrict__ runs, int nruns)
         CALL(P, w.bx, w.by, w.g & 0xffff, w.g >> 16);                                      \
     }
 template <typename T, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, 1, STR>(kPh1))) kb_phase1(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, 1, STR>(kPh1))) kb_phase1(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase1, (body_phase1<T, STR, UNI>))
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh2))) kb_phase2(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, NM, STR>(kPh2))) kb_phase2(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase2, (body_phase2<T, NM, STR, UNI>))
 template <typename T, int NM, bool STR, bool UNI>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, NM, STR>(kPh3a))) kb_phase3a(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, NM, STR>(kPh3a))) kb_phase3a(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase3a, (body_phase3a<T, NM, STR, UNI>))
+template <bool STR, bool UNI>
+__global__ void __maxnreg__(kRemap3Regs) kb_phase3a_three(const ParamsT<float>* __restrict__ runs, const BatchTile* __restrict__ work)
+{
+    typedef float T;
+    SALEC_BATCHED(phase3a, (body_phase3a<T, 3, STR, UNI>))
+}
 template <typename T>
-__global__ void __launch_bounds__(kMaxThreads) __maxnreg__((phase_regs<T, 1, false>(kPh3b))) kb_phase3b(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
+__global__ void __launch_bounds__(kMaxThreads, (phase_blocks<T, 1, false>(kPh3b))) kb_phase3b(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
 SALEC_BATCHED(phase3b, (body_phase3b<T>))
 template <typename T, int NM>
 __global__ void __launch_bounds__(kMaxThreads) kb_phase3c(const ParamsT<T>* __restrict__ runs, const BatchTile* __restrict__ work)
@@ -254,7 +270,8 @@ static cudaError_t step_impl(const ParamsT<T>& P, const dim3* blk, cudaStream_t 
     if (ev) cudaEventRecord(ev[2], s);
     k_phase2<T, NM, STR, UNI><<<grid_of(nr, nz, blk[2]), blk[2], 0, s>>>(P);
     if (ev) cudaEventRecord(ev[3], s);
-    k_phase3a<T, NM, STR, UNI><<<grid_of(nr, nz, blk[3]), blk[3], 0, s>>>(P);
+    if constexpr (sizeof(T) == 4 && NM == 3) k_phase3a_three<STR, UNI><<<grid_of(nr, nz, blk[3]), blk[3], 0, s>>>(P);
+    else k_phase3a<T, NM, STR, UNI><<<grid_of(nr, nz, blk[3]), blk[3], 0, s>>>(P);
     if (ev) cudaEventRecord(ev[4], s);
     k_phase3b<T><<<grid_of(nr + 1, nz + 1, blk[4]), blk[4], phase3b_smem<T>(blk[4]), s>>>(P);
     if (ev) cudaEventRecord(ev[5], s);
@@ -297,7 +314,8 @@ static cudaError_t batch_impl(const ParamsT<T>* runs, int nruns, const BatchTile
     if (ev) cudaEventRecord(ev[2], s);
     kb_phase2<T, NM, STR, UNI><<<ntiles[2], blk[2], 0, s>>>(runs, work[2]);
     if (ev) cudaEventRecord(ev[3], s);
-    kb_phase3a<T, NM, STR, UNI><<<ntiles[3], blk[3], 0, s>>>(runs, work[3]);
+    if constexpr (sizeof(T) == 4 && NM == 3) kb_phase3a_three<STR, UNI><<<ntiles[3], blk[3], 0, s>>>(runs, work[3]);
+    else kb_phase3a<T, NM, STR, UNI><<<ntiles[3], blk[3], 0, s>>>(runs, work[3]);
     if (ev) cudaEventRecord(ev[4], s);
     kb_phase3b<T><<<ntiles[4], blk[4], phase3b_smem<T>(blk[4]), s>>>(runs, work[4]);
     if (ev) cudaEventRecord(ev[5], s);
