@@ -17,7 +17,20 @@ constexpr int kBM = 128;          // rows of a C tile = TMEM lanes
 constexpr int kBK = 64;           // K slice per stage
 constexpr int kGemmThreads = 128;
 constexpr int kMaxNT = 128;       // widest C tile (columns = TMEM columns)
-constexpr unsigned long long kWaitNs = 2000000000ull;   // a wait on an mbarrier fails after 2 s
+// A wait on an mbarrier fails after 2 s.  Then the kernel still waits for its own copies and
+// MMAs in flight, with a limit that is as long again: the shared memory they write or read and
+// the tensor memory must not be given back under them.
+// Failure detection is tested on a build of its own (SALEC_MLP_TEST_STALL = n): the thread that
+// issues the operand copies of a tile stops after n of them, as if the others never landed, and
+// the waits are short.
+constexpr unsigned long long kDrainNs = 2000000000ull;
+#ifdef SALEC_MLP_TEST_STALL
+constexpr unsigned long long kWaitNs = 20000000ull;
+__device__ __forceinline__ bool stalled(int copies) { return copies >= SALEC_MLP_TEST_STALL; }
+#else
+constexpr unsigned long long kWaitNs = 2000000000ull;
+__device__ __forceinline__ bool stalled(int) { return false; }
+#endif
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p)
 {
@@ -79,7 +92,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity)
     return true;
 }
 
-// the same for short waits on a critical path: the clock is only read once the first polls
+// the wait for copies and MMAs in flight before their memory is given back
+__device__ __forceinline__ void mbar_drain(uint64_t* bar, uint32_t parity)
+{
+    const unsigned long long t0 = global_ns();
+    while (!mbar_try_wait(bar, parity))
+        if (global_ns() - t0 > kDrainNs) return;
+}
+
+// mbar_wait for short waits on a critical path: the clock is only read once the first polls
 // have failed (where other warps of the SM compute meanwhile, reading it between polls is the
 // better use of the issue slots: the persistent forward kernel keeps mbar_wait)
 __device__ __forceinline__ bool mbar_wait_short(uint64_t* bar, uint32_t parity)

@@ -155,8 +155,8 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_bf16(GemmArgs g)
     if (ok && issued >= 1) ok = __syncthreads_and(mbar_wait(&bars[(issued - 1) & 1], ((issued - 1) >> 1) & 1));
     if (!ok) {
         if (g.err && tid == 0) atomicOr(g.err, 1);
-        // give MMAs still in flight a bounded chance to finish before their memory goes away
-        if (issued >= 1) (void)mbar_wait(&bars[(issued - 1) & 1], ((issued - 1) >> 1) & 1);
+        // MMAs still in flight finish before their memory goes away
+        if (issued >= 1) mbar_drain(&bars[(issued - 1) & 1], ((issued - 1) >> 1) & 1);
     }
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 
@@ -233,9 +233,8 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_bf16_tma(const __grid_con
             }
         };
         bool good = true;
-        int committed = 0;              // slices whose MMAs were committed
-        const int pre = nk < ns ? nk : ns;
-        for (int kt = 0; kt < pre; ++kt) load_slice(kt);
+        int loaded = 0, committed = 0;  // slices whose copies were issued, whose MMAs were committed
+        for (; loaded < nk && loaded < ns && !stalled(loaded); ++loaded) load_slice(loaded);
         for (int kt = 0; kt < nk && good; ++kt) {
             const int st = kt % ns;
             const uint32_t par = (uint32_t)(kt / ns) & 1u;
@@ -250,10 +249,10 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_bf16_tma(const __grid_con
             }
             mma_commit(&empty[st]);
             committed = kt + 1;
-            if (kt + ns < nk) {
+            if (loaded < nk && !stalled(loaded)) {
                 // the stage is refilled once its MMAs have read it
                 if (!mbar_wait(&empty[st], par)) { good = false; break; }
-                load_slice(kt + ns);
+                load_slice(loaded++);
             }
         }
         // the last commit covers every MMA; wait for it (bounded)
@@ -261,8 +260,9 @@ __global__ void __launch_bounds__(kGemmThreads) k_gemm_bf16_tma(const __grid_con
             good = mbar_wait(&empty[(committed - 1) % ns], (uint32_t)((committed - 1) / ns) & 1u);
         if (!good) {
             if (g.err) atomicOr(g.err, 2);
-            // bounded chance for copies and MMAs still in flight to finish
-            for (int i = 0; i < ns; ++i) (void)mbar_wait(&empty[i], 0);
+            // copies and MMAs still in flight finish first
+            for (int k = committed; k < loaded; ++k) mbar_drain(&full[k % ns], (uint32_t)(k / ns) & 1u);
+            if (committed > 0) mbar_drain(&empty[(committed - 1) % ns], (uint32_t)((committed - 1) / ns) & 1u);
             ok_flag = 0;
         }
     }
@@ -298,8 +298,8 @@ constexpr uint32_t kWStageBytes = kFusedHid * kBK * 2;     // 32768
 // inputs of the tile's successor.  Jobs run in the order (pair, layer, tile) in every role.
 // mbarriers: ring stage full / empty, accumulator x complete, H_x ready (16 epilogue warps).
 // Every wait is bounded; a wait that runs out raises a shared abort flag that ends every
-// role's loop, after which the CTA waits (bounded) for its own copies and MMAs, frees its
-// tensor memory and returns.
+// role's loop.  However its loop ends, warp 0 waits for its copies and warp 1, on a barrier of
+// its own behind every MMA it issued, for its MMAs; then the tensor memory is freed.
 // ---------------------------------------------------------------------------------------
 constexpr int kPPThreads = 18 * 32;
 constexpr uint32_t kW1Bytes = kFusedHid * 16 * 2;          // layer-1 weights, K padded to 16
@@ -329,7 +329,7 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
     unsigned char* Wring = smem + 2 * kHBytes;                    // 2 stages, 1024-aligned
     unsigned char* W1s = Wring + kPPStages * kWStageBytes;        // layer-1 weights
     __shared__ __align__(16) float sbias[4 * kFusedHid + kFusedOutPad];
-    __shared__ uint64_t wfull[kPPStages], wempty[kPPStages], accfull[2], hready[2];
+    __shared__ uint64_t wfull[kPPStages], wempty[kPPStages], accfull[2], hready[2], drained;
     __shared__ uint32_t tmem_holder;
     __shared__ volatile int abort_flag;
 
@@ -338,6 +338,7 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
     if (tid == 0) {
         for (int k = 0; k < kPPStages; ++k) { mbar_init(&wfull[k], 1); mbar_init(&wempty[k], 1); }
         for (int x = 0; x < 2; ++x) { mbar_init(&accfull[x], 1); mbar_init(&hready[x], 16); }
+        mbar_init(&drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         abort_flag = 0;
     }
@@ -378,7 +379,7 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
                         if (tile_of(k, x) < 0) continue;
                         const int N = l == 4 ? kFusedOutPad : kFusedHid;
                         const CUtensorMap* map = l == 1 ? &mW2 : l == 2 ? &mW3 : l == 3 ? &mW4 : &mW5;
-                        for (int kt = 0; kt < kFusedHid / kBK; ++kt) {
+                        for (int kt = 0; kt < kFusedHid / kBK && !stalled(fills[0] + fills[1]); ++kt) {
                             if (fills[stage] > 0 && !mbar_wait_idle(&wempty[stage], (uint32_t)(fills[stage] - 1) & 1u)) {
                                 abort_flag = 1;
                                 break;
@@ -391,12 +392,12 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
                     }
             // the last copies of each stage land before the CTA's memory can go away
             for (int st = 0; st < kPPStages; ++st)
-                if (fills[st] > 0) (void)mbar_wait(&wfull[st], (uint32_t)(fills[st] - 1) & 1u);
+                if (fills[st] > 0) mbar_drain(&wfull[st], (uint32_t)(fills[st] - 1) & 1u);
         }
     } else if (warp == 1) {
         // ---- MMA issuer ----
         if (lane == 0) {
-            int used[kPPStages] = {0, 0}, hwait[2] = {0, 0}, commits[2] = {0, 0};
+            int used[kPPStages] = {0, 0}, hwait[2] = {0, 0};
             int stage = 0;
             const uint32_t w1 = smem_u32(W1s);
             for (int k = 0; k < npairs_mine && !abort_flag; ++k)
@@ -427,12 +428,10 @@ __global__ void __launch_bounds__(kPPThreads, 1) k_mlp_forward_pp(const __grid_c
                             if (abort_flag) break;
                         }
                         mma_commit(&accfull[x]);
-                        ++commits[x];
                     }
-            // MMAs still in flight finish before the tensor memory is freed
-            if (abort_flag)
-                for (int x = 0; x < 2; ++x)
-                    if (commits[x] > 0) (void)mbar_wait(&accfull[x], (uint32_t)(commits[x] - 1) & 1u);
+            // every MMA issued finishes before the tensor memory is freed
+            mma_commit(&drained);
+            mbar_drain(&drained, 0u);
         }
     } else {
         // ---- epilogue: warps 2-17; lane quarter q (TMEM lanes 32q..), column quarter cq ----

@@ -47,7 +47,8 @@ namespace mlp {
 // follows every MMA of product g - 1, the buffer's last readers.  The backward accumulators
 // alternate, since block 1 of a product may start before the epilogue of block 1 of the one
 // before has read its columns.  Every wait is bounded; one that runs out raises the abort
-// flag, every role leaves its loop, and the CTA waits (bounded) for its own copies and MMAs.
+// flag and every role leaves its loop.  However its loop ends, the TMA thread waits for its
+// copies and the MMA thread, on a barrier of its own behind every MMA it issued, for its MMAs.
 //
 // Warps: 0 TMA, 1 MMA, 2-17 epilogue (lane quarter q = warp & 3: features; samples 8 cq .. of
 // cq = (warp - 2) >> 2), 18 the training state of the step.
@@ -93,7 +94,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(const __grid_const
     unsigned char* ring = smem;
     unsigned char* op = smem + kPassStages * kSliceBytes;      // two operand buffers
     unsigned char* w1s = op + 2 * kOpBytes;
-    __shared__ uint64_t wfull[kPassStages], wempty[kPassStages], hfull[2][2], accfull[2];
+    __shared__ uint64_t wfull[kPassStages], wempty[kPassStages], hfull[2][2], accfull[2], drained;
     __shared__ uint32_t tmem_holder;
     __shared__ volatile int abort_flag;
 
@@ -112,6 +113,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(const __grid_const
             mbar_init(&hfull[k][1], 16);
             mbar_init(&accfull[k], 1);
         }
+        mbar_init(&drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         abort_flag = 0;
     }
@@ -171,12 +173,12 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(const __grid_const
                 const CUtensorMap* map = g < 5 ? &maps.w[g - 1] : &maps.wt[g - 5];
                 for (int half = 0; half < (g == 5 ? 1 : 2); ++half)
                     for (int blk = 0; blk < blocks(g); ++blk)
-                        for (int kt = 2 * half; kt < 2 * half + 2 && !abort_flag; ++kt) slice(map, kt, blk);
+                        for (int kt = 2 * half; kt < 2 * half + 2 && !abort_flag && !stalled(k); ++kt) slice(map, kt, blk);
             }
             // the last copy of each stage lands before the CTA's memory can go away
             for (int st = 0; st < kPassStages; ++st) {
                 const int uses = k > st ? (k - 1 - st) / kPassStages + 1 : 0;
-                if (uses > 0) (void)mbar_wait(&wfull[st], (uint32_t)(uses - 1) & 1u);
+                if (uses > 0) mbar_drain(&wfull[st], (uint32_t)(uses - 1) & 1u);
             }
         }
     } else if (warp == 1) {
@@ -186,7 +188,7 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(const __grid_const
             // operand (formed anew at every step they took about 280 cycles of this one thread)
             const uint32_t idesc = idesc_bf16(kBM, kNS);
             const uint64_t ring_desc = sdesc_sw128(smem_u32(ring));
-            int st = 0, commits[2] = {0, 0};
+            int st = 0;
             uint32_t par = 0, hphase[2][2] = {{0u, 0u}, {0u, 0u}};
             bool good = true;
             for (int g = 0; g < kProducts && good; ++g) {
@@ -197,7 +199,6 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(const __grid_const
                     for (int blk = 0; blk < 2; ++blk) {
                         mma_bf16(acc + blk * kNS, sdesc(smem_u32(w1s) + blk * (kBM * 16), kHidden * 16, 128), h_desc, idesc, 0u);
                         mma_commit(&accfull[blk]);
-                        ++commits[blk];
                     }
                     continue;
                 }
@@ -223,19 +224,15 @@ __global__ void __launch_bounds__(kPassThreads, 1) k_mlp_pass(const __grid_const
                                 par ^= 1u;
                             }
                         }
-                        if (good && half == halves - 1) {
-                            mma_commit(&accfull[blk]);
-                            ++commits[blk];
-                        }
+                        if (good && half == halves - 1) mma_commit(&accfull[blk]);
                     }
                 }
             }
-            if (!good) {
-                abort_flag = 1;
-                // MMAs still in flight finish before the tensor memory is freed
-                for (int blk = 0; blk < 2; ++blk)
-                    if (commits[blk] > 0) (void)mbar_wait(&accfull[blk], (uint32_t)(commits[blk] - 1) & 1u);
-            }
+            if (!good) abort_flag = 1;
+            // every MMA issued finishes before the tensor memory is freed (an epilogue warp may
+            // have given up on the last of them)
+            mma_commit(&drained);
+            mbar_drain(&drained, 0u);
         }
     } else if (warp < 18) {
         // ---- epilogues ----
@@ -485,7 +482,7 @@ __global__ void __launch_bounds__(kDwThreads) k_mlp_dw(const __grid_constant__ D
         };
         bool good = true;
         int loaded = 0, committed = 0;
-        for (; loaded < nk && loaded < kDwStages; ++loaded) load(loaded);
+        for (; loaded < nk && loaded < kDwStages && !stalled(loaded); ++loaded) load(loaded);
         for (int kt = 0; kt < nk; ++kt) {
             const int st = kt % kDwStages;
             const uint32_t par = (uint32_t)(kt / kDwStages) & 1u;
@@ -497,7 +494,7 @@ __global__ void __launch_bounds__(kDwThreads) k_mlp_dw(const __grid_constant__ D
                 mma_bf16(tmem, a_desc + off + kk * 2, b_desc + off + kk * 2, idesc, (kt > 0 || kk > 0) ? 1u : 0u);
             mma_commit(&empty[st]);
             ++committed;
-            if (loaded < nk) {
+            if (loaded < nk && !stalled(loaded)) {
                 if (!mbar_wait(&empty[st], par)) { good = false; break; }
                 load(loaded++);
             }
@@ -505,9 +502,9 @@ __global__ void __launch_bounds__(kDwThreads) k_mlp_dw(const __grid_constant__ D
         if (good) good = mbar_wait(&empty[(nk - 1) % kDwStages], (uint32_t)((nk - 1) / kDwStages) & 1u);
         if (!good) {
             if (n.err) atomicOr(n.err, 16);
-            // bounded chance for copies and MMAs still in flight to finish
-            for (int k = committed; k < loaded; ++k) (void)mbar_wait(&full[k % kDwStages], (uint32_t)(k / kDwStages) & 1u);
-            if (committed > 0) (void)mbar_wait(&empty[(committed - 1) % kDwStages], (uint32_t)((committed - 1) / kDwStages) & 1u);
+            // copies and MMAs still in flight finish first
+            for (int k = committed; k < loaded; ++k) mbar_drain(&full[k % kDwStages], (uint32_t)(k / kDwStages) & 1u);
+            if (committed > 0) mbar_drain(&empty[(committed - 1) % kDwStages], (uint32_t)((committed - 1) / kDwStages) & 1u);
             ok_flag = 0;
         }
     }
