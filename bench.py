@@ -956,7 +956,7 @@ def main():
                     "peak_nominal_kind": f"{sms} SMs (device) x {DFMA_PER_CLK_PER_SM} DFMA/clk x 2 flop x {clk:.0f} MHz",
                     "achieved": round(ach, 4) if ach else None, "frac": round(ach / fp64_gemm, 4) if ach else None,
                     "frac_of_nominal": round(ach / fp64_nominal, 4) if ach else None, **per,
-                    "traffic": tr, "traffic_kind": trk, "fp64_pipe_busy": _FP64_PIPE_BUSY.get(d),
+                    "traffic": tr, "traffic_kind": trk, "fp64_pipe_busy": _fp64_pipe_busy(d),
                     "note": "flops count 2 per DFMA and 1 per DADD/DMUL; the FP64 pipe issues every FP64 "
                             "instruction at the DFMA rate, and fp64_pipe_busy (ncu, 2000x2000) is its occupancy"}
 
@@ -1070,13 +1070,19 @@ _FUSED_FULL_SIZE: dict = {
     "fp64": {"k_rest_tiles": {"traffic": 3.0415e5}, "k_step_fused": {"traffic": 4.2143e7, "flops": 1.02645e8}},
     "fp32mix": {"k_rest_tiles": {"traffic": 1.5863e5}, "k_step_fused": {"traffic": 2.6142e7}},
 }
-# kernels changed since their counters were taken: neither DRAM traffic nor flop rates are
-# reported for them until the next capture
-_COUNTERS_STALE: dict = {"fp64": {"k_phase0", "k_phase1", "k_phase2", "k_phase3a"},
-                         "fp32mix": {"k_phase0", "k_phase2", "k_phase3a"}}
+# kernels changed since their counters were taken: neither DRAM traffic, flop rates nor the
+# FP64 pipe's share are reported for them until the next capture
+_COUNTERS_STALE: dict = {"fp64": {"k_phase0", "k_phase1", "k_phase2", "k_phase3a", "k_phase3b"},
+                         "fp32mix": {"k_phase0", "k_phase2", "k_phase3a", "k_phase3b"}}
 # Beside the copy kernel (salec_set_rest_copy mode 2) the FP64 tile kernel is another
 # instantiation (120 registers, the same arithmetic) sharing the SMs with the copies: its
 # FP64 operation count carries over, the DRAM traffic of the capture above does not.
+
+
+def _fp64_pipe_busy(kernel: str):
+    """Fraction of the FP64 pipe an FP64-form kernel keeps busy, from ncu; None without a
+    capture of the kernel as it is."""
+    return None if kernel in _COUNTERS_STALE["fp64"] else _FP64_PIPE_BUSY.get(kernel)
 
 
 def _traffic(kernel: str, prec: str, args, beside: bool = False):
