@@ -1053,13 +1053,13 @@ def main():
 # FP64 operations per cell (2 DFMA + DADD + DMUL) issued by each phase kernel of the FP64
 # form, and DRAM bytes per cell of each phase kernel, from ncu (one kernel, one launch: the
 # first timed step of the 4000 x 4000 physics at 2000 x 2000, radius 50 cells; profiles/).
-_FLOPS_PER_CELL: dict = {"k_phase0": 85.1, "k_phase1": 37.7, "k_phase2": 27.4, "k_phase3a": 51.4, "k_phase3b": 50.1, "k_phase3c": 4.8}
-_TRAFFIC_PER_CELL: dict = {"k_phase0": 57.7, "k_phase1": 72.2, "k_phase2": 75.3, "k_phase3a": 78.5, "k_phase3b": 62.8, "k_phase3c": 22.1}
-_TRAFFIC_PER_CELL_FP32MIX: dict = {"k_phase0": 27.7, "k_phase1": 30.8, "k_phase2": 40.1, "k_phase3a": 42.3, "k_phase3b": 29.6, "k_phase3c": 10.8}
+_FLOPS_PER_CELL: dict = {"k_phase0": 83.7, "k_phase1": 26.8, "k_phase2": 14.9, "k_phase3a": 36.4, "k_phase3b": 51.5, "k_phase3c": 4.8}
+_TRAFFIC_PER_CELL: dict = {"k_phase0": 57.9, "k_phase1": 72.3, "k_phase2": 75.2, "k_phase3a": 78.5, "k_phase3b": 63.0, "k_phase3c": 22.1}
+_TRAFFIC_PER_CELL_FP32MIX: dict = {"k_phase0": 27.6, "k_phase1": 30.8, "k_phase2": 40.2, "k_phase3a": 42.3, "k_phase3b": 29.6, "k_phase3c": 10.8}
 # fraction of the FP64 pipe's issue slots each FP64-form kernel keeps busy (ncu,
-# sm__pipe_fp64_cycles_active, 2000 x 2000; the fused kernels 4000 x 4000, the run's first step)
-_FP64_PIPE_BUSY: dict = {"k_phase0": 0.847, "k_phase1": 0.847, "k_phase2": 0.845, "k_phase3a": 0.847, "k_phase3b": 0.841,
-                         "k_phase3c": 0.783, "k_step_fused": 0.72, "k_rest_tiles": 0.12}
+# sm__pipe_fp64_cycles_active, 2000 x 2000; phase kernels the first timed step, fused ones the second)
+_FP64_PIPE_BUSY: dict = {"k_phase0": 0.799, "k_phase1": 0.834, "k_phase2": 0.819, "k_phase3a": 0.836, "k_phase3b": 0.841,
+                         "k_phase3c": 0.780, "k_step_fused": 0.720, "k_rest_tiles": 0.0}
 # The fused form's two kernels on the headline workload (4000 x 4000, K = 20 timed steps after
 # W = 5 warm-up steps): DRAM read + write bytes and FP64 operations per launch, the mean over
 # the 20 launches of the timed region from one-pass ncu captures of the same command
@@ -1067,15 +1067,14 @@ _FP64_PIPE_BUSY: dict = {"k_phase0": 0.847, "k_phase1": 0.847, "k_phase2": 0.845
 # for that case only.
 _FULL_SIZE_CASE = ("large_4000", 20, 5)
 _FUSED_FULL_SIZE: dict = {
-    "fp64": {"k_rest_tiles": {"traffic": 3.0415e5}, "k_step_fused": {"traffic": 4.2143e7, "flops": 1.02645e8}},
-    "fp32mix": {"k_rest_tiles": {"traffic": 1.5863e5}, "k_step_fused": {"traffic": 2.6142e7}},
+    "fp64": {"k_rest_tiles": {"traffic": 3.0449e5}, "k_step_fused": {"traffic": 4.2184e7, "flops": 1.02613e8}},
+    "fp32mix": {"k_rest_tiles": {"traffic": 1.5913e5}, "k_step_fused": {"traffic": 2.6154e7}},
 }
 # kernels changed since their counters were taken: neither DRAM traffic, flop rates nor the
 # FP64 pipe's share are reported for them until the next capture
-_COUNTERS_STALE: dict = {"fp64": {"k_phase0", "k_phase1", "k_phase2", "k_phase3a", "k_phase3b"},
-                         "fp32mix": {"k_phase0", "k_phase2", "k_phase3a", "k_phase3b"}}
+_COUNTERS_STALE: dict = {"fp64": set(), "fp32mix": set()}
 # Beside the copy kernel (salec_set_rest_copy mode 2) the FP64 tile kernel is another
-# instantiation (120 registers, the same arithmetic) sharing the SMs with the copies: its
+# kernel (at most 120 registers, the same arithmetic) sharing the SMs with the copies: its
 # FP64 operation count carries over, the DRAM traffic of the capture above does not.
 
 
