@@ -192,7 +192,10 @@ salec_status salec_step(salec_ctx* ctx, int nsteps);
  *                      Default under gravity, where no tile is quiescent and this form,
  *                      which computes no cell twice, issues fewer instructions, and in
  *                      FP64 on smaller grids.
- * Both forms compute the same cycle with the same arithmetic per cell and vertex;
+ * Both forms compute the same cycle.  Their results agree to rounding, not bit for bit: the
+ * compiler contracts multiply-adds differently in the two, and in FP64 on a uniform grid
+ * with strength the phase form adds the stresses of a column's cells before it scales them.
+ * So in FP64 a run's last bits depend on the default, hence on the grid's size.
  * salec_set_step_form returns SALEC_EINVAL for another value, SALEC_EORDER before
  * salec_finalize. */
 enum { SALEC_STEP_PHASES = 0, SALEC_STEP_FUSED = 1 };
@@ -253,8 +256,9 @@ salec_status salec_set_state(salec_ctx* ctx, const void* host, size_t bytes);
 
 /* The caller wrote the first salec_checkpoint_bytes() bytes of the state buffer itself (a
  * device-to-device copy of an earlier image, say) instead of through salec_set_state: the
- * current fields are those at the start of the buffer, and the next fused step forms the
- * Courant maximum of that state again.  SALEC_EORDER before salec_finalize. */
+ * current fields are those at the start of the buffer, and the next step, in either form or
+ * batched, forms the Courant maximum of that state again.  SALEC_EORDER before
+ * salec_finalize. */
 salec_status salec_state_changed(salec_ctx* ctx);
 
 /* Number of kernel launches one step issues (for launch accounting): in the phase form
@@ -310,7 +314,11 @@ salec_status salec_autotune(salec_ctx* ctx, int trial_steps, int* shapes_out);
  * device buffer of salec_batch_bytes() bytes (run parameter blocks and work lists).
  * salec_batch_run replays a CUDA graph of `chunk` steps until every run reaches its end
  * time or fails (status not 0), or max_steps steps; salec_batch_poll copies each run's
- * (t, dt, steps, status, t_end) into out[5 r .. 5 r + 4].  Streams: all batch work goes on the stream given here. */
+ * (t, dt, steps, status, t_end) into out[5 r .. 5 r + 4].  Streams: all batch work goes on
+ * the stream given here.  What a run's own fused steps left to do before its fields can be
+ * batched goes on the run's stream, behind them, and the batch's stream waits for it;
+ * otherwise work queued on a run's stream has to be finished before the batch steps it, and
+ * the other way round. */
 typedef struct salec_batch salec_batch;
 salec_status salec_batch_bytes(salec_ctx* const* runs, int nruns, size_t* bytes);
 salec_status salec_batch_create(salec_ctx* const* runs, int nruns, void* dev_buf, size_t bytes, void* stream,

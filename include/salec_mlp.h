@@ -21,7 +21,10 @@
  * asynchronous unless stated.  Pointers named *_dev are device pointers, *_host host
  * pointers.  Errors: SALEC_EINVAL (bad argument), SALEC_ENOMEM (buffer too small),
  * SALEC_ECUDA (CUDA error, or a tensor-core wait that ran out of time, reported by
- * salec_mlp_check); salec_mlp_last_error() gives the message. */
+ * salec_mlp_check: the kernel that gave up has then still waited for its own copies and MMAs,
+ * and what it was to write is incomplete); salec_mlp_last_error() gives the message.
+ * salec_mlp_create needs the driver's tensor-map encoder (cuTensorMapEncodeTiled, in every
+ * driver that runs this code) and returns SALEC_ECUDA without it. */
 #ifndef SALEC_MLP_H
 #define SALEC_MLP_H
 
@@ -49,9 +52,13 @@ salec_status salec_mlp_set_params(salec_mlp* mlp, const float* theta_host);
 salec_status salec_mlp_get_params(salec_mlp* mlp, float* theta_host);
 
 /* y_dev[b][o] = network(x_dev[b][:]) for b < batch <= batch_max; x_dev is batch x 5 FP32,
- * y_dev batch x 66 FP32, both row-major device arrays.  One persistent kernel runs all
- * five layers on 128-sample tiles, two per SM at a time (one on the tensor cores while the
- * other's epilogue runs), with the activations kept on chip. */
+ * y_dev batch x 66 FP32, both row-major device arrays.  One kernel runs all five layers with
+ * the activations kept on chip: up to 128 samples per SM of the device (19 456 on 152 SMs) on
+ * 32-sample tiles, one CTA each, placed on the device while the kernel before it in the
+ * stream ends (it waits for that one before it reads or writes anything); beyond that a
+ * persistent kernel on 128-sample tiles, two per SM at a time (one on the tensor cores while
+ * the other's epilogue runs), after a conversion of the inputs.  The results are bitwise the
+ * same. */
 salec_status salec_mlp_forward(salec_mlp* mlp, const float* x_dev, int batch, float* y_dev);
 
 /* Forward and backward pass against targets t_dev (batch x 66 FP32): the gradient of the
@@ -80,9 +87,9 @@ salec_status salec_mlp_train(salec_mlp* mlp, const float* x_dev, const float* t_
                              const float* lr_dev, float beta1, float beta2, float eps, double* sse_dev);
 
 /* Ensemble training: n (1..8) distinct networks trained together on the same inputs,
- * targets and learning-rate table, each step's GEMMs, Adam update and bookkeeping issued
- * as ONE launch for all members (a member index per CTA), each member with the same plan
- * and arithmetic as salec_mlp_train gives it alone, so the results are those of n separate
+ * targets and learning-rate table, each of a step's three kernels (forward and backward
+ * pass, weight gradients, their sums with the Adam update) issued as ONE launch for all
+ * members (a member index per CTA), each member with the same plan and arithmetic as salec_mlp_train gives it alone, so the results are those of n separate
  * salec_mlp_train calls.  The group holds pointers to the member contexts (which must
  * outlive it) and works on `stream` (the members' own streams are not used by group
  * calls).  salec_mlp_train_group: `steps` steps, step k with learning rate lr_dev[k]; the

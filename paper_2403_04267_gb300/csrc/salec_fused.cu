@@ -14,8 +14,9 @@
 // and then forms, for its own cells, the Courant rate of the new state (Eq. 14): the next
 // step's time step comes from the running maximum over all tiles, which a one-thread
 // kernel turns into dt before the next step starts.  Halo cells are computed by every
-// tile that needs them, from the same inputs with the same arithmetic as the phase
-// kernels, so the tiles agree on them; only the owner writes a result.  Since a tile reads
+// tile that needs them, from the same inputs with the same arithmetic, so the tiles agree on
+// them; only the owner writes a result.  (The phase kernels agree with them to rounding: in
+// FP64 on a uniform grid with strength phase 1 there adds stresses before it scales them.)  Since a tile reads
 // its neighbours' cells, the fields the step rewrites (fractions and densities, energy,
 // stress and damage, velocities, PML auxiliaries) are read from one copy and written to
 // another (ping-pong); the peak over-pressure is read and written by its owner only and
