@@ -99,16 +99,6 @@ struct Geo {
 // work on the FP64 pipe.  An upper bound in FP32 (from the high words, integer
 // instructions) decides first: warps none of whose cells can exceed the maximum seen so far
 // skip the FP64 evaluation.  The maximum that results is the same.
-__host__ __device__ __forceinline__ int high_word(double x)
-{
-#ifdef __CUDA_ARCH__
-    return __double2hiint(x);
-#else
-    long long b;
-    memcpy(&b, &x, 8);
-    return (int)(b >> 32);
-#endif
-}
 __host__ __device__ __forceinline__ float f32_of_bits(int b)
 {
 #ifdef __CUDA_ARCH__
@@ -154,11 +144,12 @@ __device__ __forceinline__ bool rate_may_raise(T2 va, T2 vb, T2 vc, T2 vd, T c2,
 // a / b with y close to 1 / b (a few units in the last place: on a non-uniform grid both y and b
 // are products, each rounded): the quotient corrected by its remainder (Markstein, IBM J. Res.
 // Dev. 34, 1990), three instructions on the FP64 pipe instead of a division's ten.  Exactly 1
-// for a == b, otherwise within 0.5 + 2^-40 units in the last place of the true quotient.
+// for a == b, otherwise within 0.5 + 2^-40 units in the last place of the true quotient; an
+// infinite a gives infinity, as the division does.
 __host__ __device__ __forceinline__ double div_by(double a, double b, double y)
 {
-    const double q = a * y;
-    return fma(fma(-q, b, a), y, q);
+    const double q = a * y, c = fma(fma(-q, b, a), y, q);
+    return (high_word(q) & 0x7ff00000) == 0x7ff00000 ? q : c;
 }
 __device__ __forceinline__ float div_by(float a, float b, float) { return a / b; }
 

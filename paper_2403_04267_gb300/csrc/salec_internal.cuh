@@ -257,6 +257,16 @@ __device__ __forceinline__ bool nonzero(float x) { return (__float_as_int(x) << 
 __device__ __forceinline__ bool below_bits(double a, double b) { return __double_as_longlong(a) < __double_as_longlong(b); }
 __device__ __forceinline__ bool below_bits(float a, float b) { return __float_as_int(a) < __float_as_int(b); }
 __device__ __forceinline__ bool warp_any(bool p);
+__host__ __device__ __forceinline__ int high_word(double x)
+{
+#ifdef __CUDA_ARCH__
+    return __double2hiint(x);
+#else
+    long long b;
+    memcpy(&b, &x, 8);
+    return (int)(b >> 32);
+#endif
+}
 
 template <typename T>
 __host__ __device__ __forceinline__ void eos_eval(const MatT<T>& m, T rho_in, T I_in, T& p_out, T& c2_out)
@@ -288,11 +298,23 @@ __host__ __device__ __forceinline__ void eos_eval(const MatT<T>& m, T rho_in, T 
     const T mu = (rho - m.rho0) * m.inv_rho0;
     // 1/rho, and 1/w0 with w0 = I / (E0 eta^2) + 1, 1/(E0 eta^2) = (rho0^2/E0) / rho^2.  The FP64
     // form takes both from one division, of which each costs ten instructions of its bound
-    // pipe: with q = rho^2 w0, 1/rho = q / (rho q) and 1/w0 = rho^2 / q
+    // pipe: with q = rho^2 w0, 1/rho = q / (rho q) and 1/w0 = rho^2 / q.  An energy or density so
+    // large that rho q might overflow takes q and rho^2 scaled down by 2^600: the sound speed of
+    // a state about to overflow must come out infinite, for the Courant step to report it
     T irho, ie, iw;
-    if (sizeof(T) == 8) {
-        const T rho2 = rho * rho;
-        const T q = I * m.rho0sq_E0 + rho2;
+    if constexpr (sizeof(T) == 8) {
+        T Is = I, rhos = rho;
+        const bool far = high_word(double(I)) >= 0x63f00000 || high_word(double(rho)) >= 0x4c700000;    // 2^576, 2^200
+#ifdef __CUDA_ARCH__
+        if (warp_any(far) && far) {
+#else
+        if (far) {
+#endif
+            Is = I * 0x1p-600;
+            rhos = rho * 0x1p-300;
+        }
+        const T rho2 = rhos * rhos;
+        const T q = Is * m.rho0sq_E0 + rho2;
         const T r = one / (rho * q);
         irho = q * r;
         ie = m.rho0sq_E0 * irho * irho;                // 1 / (E0 eta^2)

@@ -16,7 +16,7 @@ namespace salec {
 
 // Registers a thread of a phase kernel may take, set by the blocks of kMaxThreads that have to
 // fit an SM (the minimum of __launch_bounds__).  The FP64 kernels are bound by the FP64 pipe:
-// phase 0 keeps what it needs (84-94, batched 94-104, no spills; left to itself the compiler
+// phase 0 keeps what it needs (84-96, batched 94-106, no spills; left to itself the compiler
 // takes 64 and spills up to 200 bytes), the others do best as the compiler chooses (with room
 // for 128 they take 4 to 16 more, and an 800 x 800 step of two materials with strength 4 %
 // longer).  The mixed kernels are bound by
