@@ -112,8 +112,8 @@ class MLP:
 
 
 class Group:
-    """Networks (at most 8) trained together on the same data: each step's GEMMs, Adam update
-    and bookkeeping are one launch for all of them, with each member's arithmetic that of
+    """Networks (at most 8) trained together on the same data: each of a step's three kernels
+    is one launch for all of them, with each member's arithmetic that of
     MLP.train alone (salec_mlp_train_group)."""
 
     MAX = 8
@@ -357,7 +357,7 @@ class Ensemble:
             for grp in self.groups:
                 grp.train(Xd, Td, L)
         else:
-            # each member on its own stream: the members' small GEMMs run concurrently
+            # each member on its own stream: the members' kernels run concurrently
             self.streams = [torch.cuda.Stream() for _ in range(members)]
             self.nets = [train(X, Tw, steps=steps, lr=lr, seed=1000 + k, log=log, stream=self.streams[k])
                          for k in range(members)]
